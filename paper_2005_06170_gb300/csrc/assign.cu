@@ -9,8 +9,7 @@
 //   k_scatter       writes each particle as a 32-byte record (grid coordinates and the
 //                   four deposited values) at the slot an atomic increment of its key's
 //                   cursor returns: a counting sort (any order within a key).
-//   k_moments       FP64 moments (block partials) and max |q|, from velocities and masses.
-//   k_moments_final fixed-order sum of the block partials -> pkmom_moments.
+//   k_moments       FP64 moments and max |q|, from velocities and masses.
 //   k_deposit_home  (FP32, cubic, >= 1/2 particle per cell) each particle deposited
 //   + k_home_fixup  once by the tile owning its cell, halos added afterwards; otherwise
 //   k_deposit(_fx)  one CTA per output tile gathers the particles of every segment whose
@@ -24,6 +23,7 @@
 #include <utility>
 
 #include "pkmom_internal.cuh"
+#include "warp_sums.cuh"
 
 namespace pkmom {
 
@@ -71,11 +71,34 @@ cudaError_t launch_check_selftest(cudaStream_t s)
 }
 namespace {
 
+// Zeroed with the key table by the histogram's launch: the largest |q| of each field and the
+// moments' block counter.
+enum { kCtlQmax = 0, kCtlDone = 4, kCtlWords = 8 };
+
 constexpr int kHistThreads = 256;
-constexpr int kGroup = 16;  // particles per lane summed in the catalogue precision before a warp reduction
+constexpr int kMomentThreads = 256;
 
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// A 32-byte FP32 record in one 256-bit access (records_of keeps the records 32-byte aligned):
+// the lanes of a warp read records of different lines, and two 128-bit loads of each took
+// twice the wavefronts.
+__device__ __forceinline__ Record<float> load_record(const Record<float> *p)
+{
+    Record<float> r;
+    asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(r.u.x), "=f"(r.u.y), "=f"(r.u.z), "=f"(r.u.w), "=f"(r.q.x), "=f"(r.q.y), "=f"(r.q.z), "=f"(r.q.w)
+        : "l"(p));
+    return r;
+}
+__device__ __forceinline__ void store_record(Record<float> *p, const Record<float> &r)
+{
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(r.u.x), "f"(r.u.y),
+                 "f"(r.u.z), "f"(r.u.w), "f"(r.q.x), "f"(r.q.y), "f"(r.q.z), "f"(r.q.w)
+                 : "memory");
+}
+__device__ __forceinline__ void store_record(Record<double> *p, const Record<double> &r) { *p = r; }
 
 // floor(u) wrapped into [0, ng); false for non-finite or huge |u|.
 template <typename T>
@@ -143,22 +166,6 @@ k_hist(const T *__restrict__ x, const T *__restrict__ y, const T *__restrict__ z
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += 2 * step) {
         one(i);
         if (i + step < n) one(i + step);
-    }
-}
-
-__global__ void k_moments_final(const double *__restrict__ partials, int nblocks, int64_t n_particles,
-                                double *__restrict__ out)
-{
-    // one warp per moment value, fixed summation order
-    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (k >= kMomentVals) return;
-    double s = 0.0;
-    for (int b = lane; b < nblocks; b += 32) s += partials[static_cast<int64_t>(b) * kMomentWords + k];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) out[k] = s;
-    if (k == 0 && lane == 0) {
-        out[kMomentVals] = static_cast<double>(n_particles);
-        out[kMomentVals + 1] = 0.0;
     }
 }
 
@@ -279,170 +286,203 @@ k_scan_apply(uint32_t *__restrict__ counts, int64_t nkeys, const uint32_t *__res
 }
 
 // ------------------------------------------------------------------ moments
-// The catalogue moments and the largest |q| of each deposited field, from velocities
-// and masses alone: each lane sums kGroup particles in the catalogue precision (four
-// per iteration, loads issued first), the warp adds its lanes' group sums (shuffles)
-// and lane 0 adds them to FP64 accumulators, so that FP64 work is one add per value
-// per 32 * kGroup particles; block sums go to partials[block] (k_moments_final).
-template <typename T>
-__global__ void __launch_bounds__(256)
-k_moments(const T *__restrict__ vx, const T *__restrict__ vy, const T *__restrict__ vz, const T *__restrict__ mass,
-          int64_t stride, int64_t n, double *__restrict__ partials, unsigned *__restrict__ qmax_bits)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __shared__ double s_part[256 / 32][kMomentVals];  // per-warp FP64 sums
-    if (lane < kMomentVals) s_part[warp][lane] = 0.0;
-    __syncwarp();
-    float qmax[4] = {0.f, 0.f, 0.f, 0.f};
-    T grp[kMomentVals];
+// Sums of one lane's particles, in a fixed order: FP32 catalogues in compensated (Kahan) FP32
+// pairs, so that neither FP64 work nor a warp reduction runs inside the loop; FP64 ones in
+// plain FP64. With unit masses the sums of m and m^2 are the particle count and those of
+// m^2 v are those of m v, so only nine of the fourteen are kept.
+template <typename T, bool MASS>
+struct LaneMoments {
+    static constexpr int NV = MASS ? kMomentVals : 9;
+    T sum[NV], cmp[NV];  // the sum of a value is sum - cmp
+    T qmax[4];
+    __device__ __forceinline__ LaneMoments()
+    {
 #pragma unroll
-    for (int k = 0; k < kMomentVals; ++k) grp[k] = T(0);
-    int gcount = 0;
-    const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    auto flush = [&]() {
+        for (int k = 0; k < NV; ++k) sum[k] = T(0), cmp[k] = T(0);
 #pragma unroll
-        for (int k = 0; k < kMomentVals; ++k) {
-            T v = grp[k];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) s_part[warp][k] += static_cast<double>(v);
-            grp[k] = T(0);
+        for (int f = 0; f < 4; ++f) qmax[f] = T(0);
+    }
+    __device__ __forceinline__ void put(int k, T x)
+    {
+        if constexpr (sizeof(T) == 4) {
+            const T y = __fsub_rn(x, cmp[k]);
+            const T t = __fadd_rn(sum[k], y);
+            cmp[k] = __fsub_rn(__fsub_rn(t, sum[k]), y);
+            sum[k] = t;
+        } else {
+            sum[k] += x;
         }
-    };
-    auto add = [&](T m, T v0, T v1, T v2) {
-        const T m2 = m * m;
-        qmax[0] = fmaxf(qmax[0], static_cast<float>(fabs(m)));
-        qmax[1] = fmaxf(qmax[1], static_cast<float>(fabs(m * v0)));
-        qmax[2] = fmaxf(qmax[2], static_cast<float>(fabs(m * v1)));
-        qmax[3] = fmaxf(qmax[3], static_cast<float>(fabs(m * v2)));
-        grp[0] += m;
-        grp[1] += m2;
-        grp[2] += m * v0;
-        grp[3] += m * v1;
-        grp[4] += m * v2;
-        grp[5] += m2 * v0;
-        grp[6] += m2 * v1;
-        grp[7] += m2 * v2;
-        grp[8] += m2 * v0 * v0;
-        grp[9] += m2 * v1 * v1;
-        grp[10] += m2 * v2 * v2;
-        grp[11] += m2 * v0 * v1;
-        grp[12] += m2 * v0 * v2;
-        grp[13] += m2 * v1 * v2;
-    };
-    // warp-uniform loop: every lane runs the same iterations (shuffles inside)
-    for (int64_t wb = static_cast<int64_t>(blockIdx.x) * blockDim.x + (threadIdx.x & ~31); wb < n; wb += 4 * step) {
+    }
+    __device__ __forceinline__ void add(T m, T v0, T v1, T v2)
+    {
+        if constexpr (MASS) {
+            const T m2 = m * m, p0 = m * v0, p1 = m * v1, p2 = m * v2;
+            top(0, m), top(1, p0), top(2, p1), top(3, p2);
+            put(0, m);
+            put(1, m2);
+            put(2, p0);
+            put(3, p1);
+            put(4, p2);
+            put(5, m2 * v0);
+            put(6, m2 * v1);
+            put(7, m2 * v2);
+            put(8, m2 * v0 * v0);
+            put(9, m2 * v1 * v1);
+            put(10, m2 * v2 * v2);
+            put(11, m2 * v0 * v1);
+            put(12, m2 * v0 * v2);
+            put(13, m2 * v1 * v2);
+        } else {
+            top(1, v0), top(2, v1), top(3, v2);
+            put(0, v0);
+            put(1, v1);
+            put(2, v2);
+            put(3, v0 * v0);
+            put(4, v1 * v1);
+            put(5, v2 * v2);
+            put(6, v0 * v1);
+            put(7, v0 * v2);
+            put(8, v1 * v2);
+        }
+    }
+    __device__ __forceinline__ void top(int f, T x)
+    {
+        if constexpr (sizeof(T) == 4) qmax[f] = fmaxf(qmax[f], fabsf(x));
+        else qmax[f] = fabs(x) > qmax[f] ? fabs(x) : qmax[f];
+    }
+};
+
+// The moments of the catalogue from the lanes' sums: warp reduce-scatters (float pairs, so
+// that a warp does two FP64 adds instead of 70: FP64 runs at under two lanes a clock per SM
+// on this part), one partial per block, and the last block to finish adds the partials in a
+// fixed order into out (pkmom_moments). done: a zeroed counter. As FP64 butterflies in 1216
+// blocks and a separate kernel the same sums took 80 us whatever the catalogue's size.
+template <typename T, bool MASS>
+__device__ __forceinline__ void finish_moments(LaneMoments<T, MASS> &lm, int64_t n, double *__restrict__ partials,
+                                               unsigned *__restrict__ qmax_bits, unsigned *__restrict__ done,
+                                               double *__restrict__ out)
+{
+    constexpr int NV = LaneMoments<T, MASS>::NV, NG = (NV + 7) / 8;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    __shared__ double s_part[kMomentThreads / 32][8 * NG];
+    __shared__ bool s_last;
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+        double x;
+        if constexpr (sizeof(T) == 4) {
+            T hi[8], lo[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                hi[k] = 8 * g + k < NV ? lm.sum[8 * g + k < NV ? 8 * g + k : 0] : T(0);
+                lo[k] = 8 * g + k < NV ? -lm.cmp[8 * g + k < NV ? 8 * g + k : 0] : T(0);
+            }
+            x = warp_scatter_sum8(hi, lo);
+        } else {
+            double v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = 8 * g + k < NV ? lm.sum[8 * g + k < NV ? 8 * g + k : 0] : T(0);
+            x = warp_scatter_sum8(v);
+        }
+        if ((lane & 3) == 0) s_part[warp][8 * g + (lane >> 2)] = x;
+    }
+    if constexpr (!MASS) lm.qmax[0] = T(1);
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        // non-negative floats order like their bit patterns
+        const unsigned bits = __reduce_max_sync(0xffffffffu, __float_as_uint(static_cast<float>(lm.qmax[f])));
+        if (lane == 0) atomicMax(qmax_bits + f, bits);
+    }
+    __syncthreads();
+    if (threadIdx.x < NV) {
+        double total = 0.0;
+        for (int w = 0; w < nw; ++w) total += s_part[w][threadIdx.x];
+        partials[static_cast<int64_t>(blockIdx.x) * kMomentWords + threadIdx.x] = total;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // value k by warps k, k + nw, ...; without masses: m v, then m^2 v v^T
+    for (int k = warp; k < NV; k += nw) {
+        double x = 0.0;
+        for (int b = lane; b < static_cast<int>(gridDim.x); b += 32)
+            x += __ldcg(partials + static_cast<int64_t>(b) * kMomentWords + k);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane != 0) continue;
+        if constexpr (MASS) out[k] = x;
+        else if (k < 3) out[2 + k] = x, out[5 + k] = x;
+        else out[5 + k] = x;
+    }
+    if (threadIdx.x == 0) {
+        if constexpr (!MASS) out[0] = out[1] = static_cast<double>(n);
+        out[kMomentVals] = static_cast<double>(n);
+        out[kMomentVals + 1] = 0.0;
+    }
+}
+
+// The catalogue moments and the largest |q| of each deposited field, from velocities
+// and masses alone (mass may be null only with MASS false).
+template <typename T, bool MASS>
+__global__ void __launch_bounds__(kMomentThreads)
+k_moments(const T *__restrict__ vx, const T *__restrict__ vy, const T *__restrict__ vz, const T *__restrict__ mass,
+          int64_t stride, int64_t n, double *__restrict__ partials, unsigned *__restrict__ qmax_bits,
+          unsigned *__restrict__ done, double *__restrict__ out)
+{
+    LaneMoments<T, MASS> lm;
+    const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i0 < n; i0 += 4 * step) {
         T m[4], a[4], b[4], c[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int64_t i = wb + k * step + lane;
+            const int64_t i = i0 + k * step;
             const bool ok = i < n;
             const int64_t j = ok ? i * stride : 0;
-            m[k] = ok ? (mass ? mass[i] : T(1)) : T(0);  // absent particles add nothing
+            m[k] = T(0);
+            if constexpr (MASS) m[k] = ok ? mass[i] : T(0);  // absent particles add nothing
             a[k] = ok ? vx[j] : T(0);
             b[k] = ok ? vy[j] : T(0);
             c[k] = ok ? vz[j] : T(0);
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) add(m[k], a[k], b[k], c[k]);
-        gcount += 4;
-        if (gcount >= kGroup) {
-            flush();
-            gcount = 0;
-        }
+        for (int k = 0; k < 4; ++k) lm.add(m[k], a[k], b[k], c[k]);
     }
-    flush();
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-        // non-negative floats order like their bit patterns
-        const unsigned bits = __reduce_max_sync(0xffffffffu, __float_as_uint(qmax[f]));
-        if (lane == 0) atomicMax(qmax_bits + f, bits);
-    }
-    __syncthreads();
-    if (threadIdx.x < kMomentVals) {
-        double sum = 0.0;
-        for (int w = 0; w < 256 / 32; ++w) sum += s_part[w][threadIdx.x];
-        partials[static_cast<int64_t>(blockIdx.x) * kMomentWords + threadIdx.x] = sum;
-    }
+    finish_moments<T, MASS>(lm, n, partials, qmax_bits, done, out);
 }
 
 // FP32 interleaved (n, 3) velocities, 16-byte aligned: four particles per thread read
 // as three 128-bit loads ((v0x v0y v0z v1x) (v1y v1z v2x v2y) (v2z v3x v3y v3z)), and
-// four masses as one. The same sums as k_moments, kept by each lane in compensated
-// (Kahan) FP32 pairs over all of its particles, so that no warp reduction waits inside
-// the loop; each lane's pairs go to FP64 once at the end and are summed in a fixed
-// order. The n % 4 last particles are added by the first lanes of block 0.
-__global__ void __launch_bounds__(256)
-k_moments_v3(const float *__restrict__ v, const float *__restrict__ mass, int64_t n,
-             double *__restrict__ partials, unsigned *__restrict__ qmax_bits)
+// four masses as one. The n % 4 last particles are added by the first lanes of block 0.
+template <bool MASS>
+__global__ void __launch_bounds__(kMomentThreads)
+k_moments_v3(const float *__restrict__ v, const float *__restrict__ mass, int64_t n, double *__restrict__ partials,
+             unsigned *__restrict__ qmax_bits, unsigned *__restrict__ done, double *__restrict__ out)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __shared__ double s_part[256 / 32][kMomentVals];
-    float qmax[4] = {0.f, 0.f, 0.f, 0.f};
-    float sum[kMomentVals], cmp[kMomentVals];  // the sum of a value is sum - cmp
-#pragma unroll
-    for (int k = 0; k < kMomentVals; ++k) sum[k] = 0.f, cmp[k] = 0.f;
+    LaneMoments<float, MASS> lm;
     const int64_t nq = n / 4;
     const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x;
     const float4 *v4 = reinterpret_cast<const float4 *>(v);
     const float4 *m4 = reinterpret_cast<const float4 *>(mass);
-    auto kahan = [&](int k, float x) {
-        const float y = __fsub_rn(x, cmp[k]);
-        const float t = __fadd_rn(sum[k], y);
-        cmp[k] = __fsub_rn(__fsub_rn(t, sum[k]), y);
-        sum[k] = t;
-    };
-    auto add = [&](float m, float v0, float v1, float v2) {
-        const float m2 = m * m;
-        qmax[0] = fmaxf(qmax[0], fabsf(m));
-        qmax[1] = fmaxf(qmax[1], fabsf(m * v0));
-        qmax[2] = fmaxf(qmax[2], fabsf(m * v1));
-        qmax[3] = fmaxf(qmax[3], fabsf(m * v2));
-        kahan(0, m);
-        kahan(1, m2);
-        kahan(2, m * v0);
-        kahan(3, m * v1);
-        kahan(4, m * v2);
-        kahan(5, m2 * v0);
-        kahan(6, m2 * v1);
-        kahan(7, m2 * v2);
-        kahan(8, m2 * v0 * v0);
-        kahan(9, m2 * v1 * v1);
-        kahan(10, m2 * v2 * v2);
-        kahan(11, m2 * v0 * v1);
-        kahan(12, m2 * v0 * v2);
-        kahan(13, m2 * v1 * v2);
-    };
     for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < nq; q += step) {
         const float4 a = v4[3 * q], b = v4[3 * q + 1], c = v4[3 * q + 2];
-        const float4 mm = mass ? m4[q] : make_float4(1.f, 1.f, 1.f, 1.f);
-        add(mm.x, a.x, a.y, a.z);
-        add(mm.y, a.w, b.x, b.y);
-        add(mm.z, b.z, b.w, c.x);
-        add(mm.w, c.y, c.z, c.w);
+        float4 mm = make_float4(1.f, 1.f, 1.f, 1.f);
+        if constexpr (MASS) mm = m4[q];
+        lm.add(mm.x, a.x, a.y, a.z);
+        lm.add(mm.y, a.w, b.x, b.y);
+        lm.add(mm.z, b.z, b.w, c.x);
+        lm.add(mm.w, c.y, c.z, c.w);
     }
-    if (blockIdx.x == 0 && warp == 0) {
-        const int64_t i = 4 * nq + lane;
-        if (i < n) add(mass ? mass[i] : 1.f, v[3 * i], v[3 * i + 1], v[3 * i + 2]);
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        const int64_t i = 4 * nq + threadIdx.x;
+        if (i < n) {
+            float m = 1.f;
+            if constexpr (MASS) m = mass[i];
+            lm.add(m, v[3 * i], v[3 * i + 1], v[3 * i + 2]);
+        }
     }
-#pragma unroll
-    for (int k = 0; k < kMomentVals; ++k) {
-        double x = static_cast<double>(sum[k]) - static_cast<double>(cmp[k]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == 0) s_part[warp][k] = x;
-    }
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-        const unsigned bits = __reduce_max_sync(0xffffffffu, __float_as_uint(qmax[f]));
-        if (lane == 0) atomicMax(qmax_bits + f, bits);
-    }
-    __syncthreads();
-    if (threadIdx.x < kMomentVals) {
-        double total = 0.0;
-        for (int w = 0; w < 256 / 32; ++w) total += s_part[w][threadIdx.x];
-        partials[static_cast<int64_t>(blockIdx.x) * kMomentWords + threadIdx.x] = total;
-    }
+    finish_moments<float, MASS>(lm, n, partials, qmax_bits, done, out);
 }
 
 // ------------------------------------------------------------------ scatter
@@ -469,7 +509,7 @@ k_scatter(const T *__restrict__ x, const T *__restrict__ y, const T *__restrict_
         Record<T> r;
         r.u = Vec4<T>{u0 - floor(u0), u1 - floor(u1), u2 - floor(u2), pack_cell<T>(c0, c1, c2)};
         r.q = Vec4<T>{m, m * vx[j], m * vy[j], m * vz[j]};
-        rec[dst] = r;
+        store_record(rec + dst, r);
     }
 }
 
@@ -2114,15 +2154,24 @@ uint32_t *key_table(const AssignPlan &pl, void *scratch)
     return reinterpret_cast<uint32_t *>(static_cast<char *>(scratch) + pl.off_counts) + 4;
 }
 
-cudaError_t launch_hist_moments(const pkmom_catalog &cat, const AssignPlan &pl, double box_L, void *scratch,
-                                int *err_flag, cudaStream_t s, LaunchStats &st)
+// The sorted records: on a 32-byte boundary (the scratch is 16-byte aligned; plan_assign
+// leaves room for the shift).
+void *records_of(const AssignPlan &pl, void *scratch)
+{
+    const uintptr_t a = reinterpret_cast<uintptr_t>(static_cast<char *>(scratch) + pl.off_records);
+    return reinterpret_cast<void *>((a + 31) & ~uintptr_t(31));
+}
+unsigned *control_words(const AssignPlan &pl, void *scratch)
+{
+    return reinterpret_cast<unsigned *>(static_cast<char *>(scratch) + pl.off_control);
+}
+
+cudaError_t launch_hist(const pkmom_catalog &cat, const AssignPlan &pl, double box_L, void *scratch, int *err_flag,
+                        cudaStream_t s, LaunchStats &st)
 {
     char *sc = static_cast<char *>(scratch);
     uint32_t *counts = key_table(pl, scratch);
-    auto *qmax = reinterpret_cast<unsigned *>(sc + pl.off_qmax);
-    cudaError_t e = cudaMemsetAsync(sc + pl.off_counts, 0, key_table_bytes(pl.nkeys), s);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(qmax, 0, 4 * sizeof(unsigned), s);  // maxima taken by the scatter
+    cudaError_t e = cudaMemsetAsync(sc + pl.off_counts, 0, pl.off_records - pl.off_counts, s);
     if (e != cudaSuccess) return e;
     const double scale = static_cast<double>(pl.ng) / box_L;
     if (pl.prec == PKMOM_F32) {
@@ -2138,15 +2187,7 @@ cudaError_t launch_hist_moments(const pkmom_catalog &cat, const AssignPlan &pl, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_moments_final(const AssignPlan &pl, int64_t n, void *scratch, double *moments_dev,
-                                 cudaStream_t s, LaunchStats &st)
-{
-    char *sc = static_cast<char *>(scratch);
-    auto *partials = reinterpret_cast<const double *>(sc + pl.off_partials);
-    k_moments_final<<<1, 32 * kMomentVals, 0, s>>>(partials, pl.hist_blocks, n, moments_dev);
-    st.launches++;
-    return cudaGetLastError();
-}
+size_t control_bytes() { return kCtlWords * sizeof(unsigned); }
 
 cudaError_t launch_scan(const AssignPlan &pl, void *scratch, cudaStream_t s, LaunchStats &st)
 {
@@ -2161,40 +2202,47 @@ cudaError_t launch_scan(const AssignPlan &pl, void *scratch, cudaStream_t s, Lau
     return cudaGetLastError();
 }
 
-cudaError_t launch_scatter(const pkmom_catalog &cat, const AssignPlan &pl, double box_L, void *scratch,
-                           cudaStream_t s, LaunchStats &st)
+namespace {
+template <typename T>
+void scatter_and_moments(const pkmom_catalog &cat, const AssignPlan &pl, T scale, void *scratch, double *moments_dev,
+                         cudaStream_t s)
 {
     char *sc = static_cast<char *>(scratch);
-    uint32_t *cursor = key_table(pl, scratch);
+    unsigned *ctl = control_words(pl, scratch);
+    const T *vx = tp<T>(cat.vx), *vy = tp<T>(cat.vy), *vz = tp<T>(cat.vz), *mass = tp<T>(cat.mass);
+    k_scatter<T><<<pl.hist_blocks, 256, 0, s>>>(tp<T>(cat.x), tp<T>(cat.y), tp<T>(cat.z), vx, vy, vz, mass, cat.stride,
+                                                cat.n, scale, pl.ng, pl.sshift, key_table(pl, scratch),
+                                                static_cast<Record<T> *>(records_of(pl, scratch)));
     auto *partials = reinterpret_cast<double *>(sc + pl.off_partials);
-    auto *qmax = reinterpret_cast<unsigned *>(sc + pl.off_qmax);
-    const double scale = static_cast<double>(pl.ng) / box_L;
-    const unsigned blocks = pl.hist_blocks;  // k_moments: one partial per block
-    if (pl.prec == PKMOM_F32) {
-        k_scatter<float><<<blocks, 256, 0, s>>>(tp<float>(cat.x), tp<float>(cat.y), tp<float>(cat.z),
-                                                tp<float>(cat.vx), tp<float>(cat.vy), tp<float>(cat.vz),
-                                                tp<float>(cat.mass), cat.stride, cat.n, static_cast<float>(scale),
-                                                pl.ng, pl.sshift, cursor,
-                                                reinterpret_cast<Record<float> *>(sc + pl.off_records));
-        const char *bv = static_cast<const char *>(cat.vx);
-        const bool v3 = cat.stride == 3 && static_cast<const char *>(cat.vy) == bv + 4 &&
-                        static_cast<const char *>(cat.vz) == bv + 8 && reinterpret_cast<uintptr_t>(bv) % 16 == 0 &&
-                        (!cat.mass || reinterpret_cast<uintptr_t>(cat.mass) % 16 == 0);
-        if (v3)
-            k_moments_v3<<<blocks, 256, 0, s>>>(tp<float>(cat.vx), tp<float>(cat.mass), cat.n, partials, qmax);
-        else
-            k_moments<float><<<blocks, 256, 0, s>>>(tp<float>(cat.vx), tp<float>(cat.vy), tp<float>(cat.vz),
-                                                    tp<float>(cat.mass), cat.stride, cat.n, partials, qmax);
-    } else {
-        k_scatter<double><<<blocks, 256, 0, s>>>(tp<double>(cat.x), tp<double>(cat.y), tp<double>(cat.z),
-                                                 tp<double>(cat.vx), tp<double>(cat.vy), tp<double>(cat.vz),
-                                                 tp<double>(cat.mass), cat.stride, cat.n, scale, pl.ng, pl.sshift,
-                                                 cursor, reinterpret_cast<Record<double> *>(sc + pl.off_records));
-        k_moments<double><<<blocks, 256, 0, s>>>(tp<double>(cat.vx), tp<double>(cat.vy), tp<double>(cat.vz),
-                                                 tp<double>(cat.mass), cat.stride, cat.n, partials, qmax);
+    // four particles a thread at least: the blocks' sums are FP64 work of the last block
+    const int64_t want = (cat.n + 4 * kMomentThreads - 1) / (4 * kMomentThreads);
+    const unsigned blocks = static_cast<unsigned>(std::min<int64_t>(want, pl.hist_blocks / 2));
+    unsigned *qmax = ctl + kCtlQmax, *done = ctl + kCtlDone;
+    if constexpr (sizeof(T) == 4) {
+        const bool v3 = cat.stride == 3 && vy == vx + 1 && vz == vx + 2 && reinterpret_cast<uintptr_t>(vx) % 16 == 0 &&
+                        reinterpret_cast<uintptr_t>(mass) % 16 == 0;
+        if (v3) {
+            if (mass) k_moments_v3<true><<<blocks, kMomentThreads, 0, s>>>(vx, mass, cat.n, partials, qmax, done, moments_dev);
+            else k_moments_v3<false><<<blocks, kMomentThreads, 0, s>>>(vx, mass, cat.n, partials, qmax, done, moments_dev);
+            return;
+        }
     }
-    st.launches++;
-    st.launches++;
+    if (mass)
+        k_moments<T, true><<<blocks, kMomentThreads, 0, s>>>(vx, vy, vz, mass, cat.stride, cat.n, partials, qmax, done,
+                                                             moments_dev);
+    else
+        k_moments<T, false><<<blocks, kMomentThreads, 0, s>>>(vx, vy, vz, mass, cat.stride, cat.n, partials, qmax, done,
+                                                              moments_dev);
+}
+}  // namespace
+
+cudaError_t launch_scatter(const pkmom_catalog &cat, const AssignPlan &pl, double box_L, void *scratch,
+                           double *moments_dev, cudaStream_t s, LaunchStats &st)
+{
+    const double scale = static_cast<double>(pl.ng) / box_L;
+    if (pl.prec == PKMOM_F32) scatter_and_moments<float>(cat, pl, static_cast<float>(scale), scratch, moments_dev, s);
+    else scatter_and_moments<double>(cat, pl, scale, scratch, moments_dev, s);
+    st.launches += 2;
     return cudaGetLastError();
 }
 
@@ -2205,11 +2253,10 @@ bool batchable_deposit(const AssignPlan &pl)
 
 FxJob deposit_job(const AssignPlan &pl, void *scratch, void *grids)
 {
-    char *sc = static_cast<char *>(scratch);
     FxJob j{};
-    j.rec = reinterpret_cast<const Record<float> *>(sc + pl.off_records);
+    j.rec = static_cast<const Record<float> *>(records_of(pl, scratch));
     j.offsets = key_table(pl, scratch) - 1;
-    j.qmax = reinterpret_cast<const unsigned *>(sc + pl.off_qmax);
+    j.qmax = control_words(pl, scratch);
     j.grids = static_cast<float *>(grids);
     j.grid_elems = static_cast<int64_t>(pl.ng) * pl.ng * (pl.ng + 2);
     j.ng = pl.ng;
@@ -2248,8 +2295,8 @@ cudaError_t launch_deposit(const AssignPlan &pl, void *scratch, void *grids, cud
 {
     char *sc = static_cast<char *>(scratch);
     const uint32_t *offsets = key_table(pl, scratch) - 1;  // offset[0..nkeys] after the scatter
-    auto *qmax = reinterpret_cast<const unsigned *>(sc + pl.off_qmax);
-    const void *rec = sc + pl.off_records;
+    const unsigned *qmax = control_words(pl, scratch);
+    const void *rec = records_of(pl, scratch);
     float *halo = pl.off_halo ? reinterpret_cast<float *>(sc + pl.off_halo) : nullptr;
     cudaError_t e;
     if (pl.bl_radius > 0) {

@@ -200,14 +200,14 @@ AssignPlan plan_assign(const pkmom_params &p, int64_t n, int num_sms, int tile_o
     size_t off = 0;
     pl.off_counts = off;
     off = align_up(off + key_table_bytes(pl.nkeys));
+    pl.off_control = off;  // [off_counts, off_records) is zeroed by every assignment
+    off = align_up(off + control_bytes());
     pl.off_records = off;
-    off = align_up(off + size_t(n) * rec);
+    off = align_up(off + size_t(n) * rec + 32);  // records start on a 32-byte boundary
     pl.off_partials = off;
     off = align_up(off + size_t(pl.hist_blocks) * kMomentWords * 8);
     pl.off_blocksums = off;
     off = align_up(off + size_t(pl.scan_blocks + 1) * 4);
-    pl.off_qmax = off;
-    off = align_up(off + 4 * sizeof(unsigned));
     if (pl.tile == kHomeTile && p.order == 4) {
         pl.off_halo = off;
         off = align_up(off + home_halo_bytes(p.ng));
@@ -550,7 +550,7 @@ pkmom_status pkmom_assign(pkmom_ctx *ctx, const pkmom_catalog *cat, const pkmom_
     cudaStream_t st = as_stream(stream);
     {
         StageTimer t(ctx, PKMOM_STAGE_HIST, st);
-        PK_CUDA(launch_hist_moments(*cat, pl, p->box_L, scratch, ctx->d_err, st, ctx->st), "histogram");
+        PK_CUDA(launch_hist(*cat, pl, p->box_L, scratch, ctx->d_err, st, ctx->st), "histogram");
     }
     {
         StageTimer t(ctx, PKMOM_STAGE_SCAN, st);
@@ -558,9 +558,8 @@ pkmom_status pkmom_assign(pkmom_ctx *ctx, const pkmom_catalog *cat, const pkmom_
     }
     {
         StageTimer t(ctx, PKMOM_STAGE_SCATTER, st);
-        PK_CUDA(launch_scatter(*cat, pl, p->box_L, scratch, st, ctx->st), "scatter and moments");
-        PK_CUDA(launch_moments_final(pl, cat->n, scratch, static_cast<double *>(moments_dev), st, ctx->st),
-                "moments");
+        PK_CUDA(launch_scatter(*cat, pl, p->box_L, scratch, static_cast<double *>(moments_dev), st, ctx->st),
+                "scatter and moments");
     }
     {
         StageTimer t(ctx, PKMOM_STAGE_DEPOSIT, st);
@@ -614,7 +613,7 @@ pkmom_status pkmom_spectra(pkmom_ctx *ctx, const pkmom_params *p, const void *gr
     }
     {
         StageTimer tm(ctx, PKMOM_STAGE_FINAL, st);
-        PK_CUDA(launch_finalize(*t, *p, static_cast<const double *>(moments_dev), out_dev, st, ctx->st, true),
+        PK_CUDA(launch_finalize(*t, *p, static_cast<const double *>(moments_dev), out_dev, st, ctx->st),
                 "finalize");
     }
     return PKMOM_OK;
@@ -769,21 +768,18 @@ pkmom_status pkmom_wait(pkmom_ctx *ctx, int64_t ticket)
 namespace {
 struct BatchLayout {
     size_t counter = 0, total = 0;
-    std::vector<size_t> partials, sums;  // offsets per item (FP32 items), else unused
+    std::vector<size_t> partials;  // offsets per item (FP32 items), else unused
 };
 BatchLayout batch_layout(int n, const pkmom_batch_item *items)
 {
     BatchLayout L;
     size_t off = align_up(sizeof(unsigned long long));
     L.partials.assign(n, 0);
-    L.sums.assign(n, 0);
     for (int k = 0; k < n; ++k) {
         const pkmom_params &p = items[k].p;
         if (p.precision != PKMOM_F32) continue;
         L.partials[k] = off;
         off = align_up(off + size_t(p.ng) * p.nbins * kBinVals * sizeof(double));
-        L.sums[k] = off;
-        off = align_up(off + size_t(kBinVals) * p.nbins * sizeof(double));
     }
     L.total = off;
     return L;
@@ -834,7 +830,7 @@ pkmom_status pkmom_estimate_batch(pkmom_ctx *ctx, int n, const pkmom_batch_item 
     {
         StageTimer t(ctx, PKMOM_STAGE_HIST, st);
         for (int k = 0; k < n; ++k)
-            PK_CUDA(launch_hist_moments(items[k].cat, plans[k], items[k].p.box_L, items[k].scratch, ctx->d_err, st,
+            PK_CUDA(launch_hist(items[k].cat, plans[k], items[k].p.box_L, items[k].scratch, ctx->d_err, st,
                                         ctx->st),
                     "histogram");
     }
@@ -845,11 +841,9 @@ pkmom_status pkmom_estimate_batch(pkmom_ctx *ctx, int n, const pkmom_batch_item 
     {
         StageTimer t(ctx, PKMOM_STAGE_SCATTER, st);
         for (int k = 0; k < n; ++k) {
-            PK_CUDA(launch_scatter(items[k].cat, plans[k], items[k].p.box_L, items[k].scratch, st, ctx->st),
+            PK_CUDA(launch_scatter(items[k].cat, plans[k], items[k].p.box_L, items[k].scratch,
+                                   static_cast<double *>(items[k].moments_dev), st, ctx->st),
                     "scatter and moments");
-            PK_CUDA(launch_moments_final(plans[k], items[k].cat.n, items[k].scratch,
-                                         static_cast<double *>(items[k].moments_dev), st, ctx->st),
-                    "moments");
         }
     }
     {
@@ -869,7 +863,7 @@ pkmom_status pkmom_estimate_batch(pkmom_ctx *ctx, int n, const pkmom_batch_item 
         bb.counter = reinterpret_cast<unsigned *>(counter);  // the deposit's counter, free again
         std::vector<const SpectraTables *> btabs;
         std::vector<const pkmom_params *> bpar;
-        std::vector<double *> bsums, bout;
+        std::vector<double *> bout;
         for (int k = 0; k < n; ++k) {
             const pkmom_batch_item &it = items[k];
             if (it.p.precision != PKMOM_F32) {
@@ -877,7 +871,7 @@ pkmom_status pkmom_estimate_batch(pkmom_ctx *ctx, int n, const pkmom_batch_item 
                                           ctx->st),
                         "binning");
                 PK_CUDA(launch_finalize(*tabs[k], it.p, static_cast<const double *>(it.moments_dev), it.out_dev, st,
-                                        ctx->st, true),
+                                        ctx->st),
                         "finalize");
                 continue;
             }
@@ -892,12 +886,10 @@ pkmom_status pkmom_estimate_batch(pkmom_ctx *ctx, int n, const pkmom_batch_item 
             j.nbins = it.p.nbins;
             btabs.push_back(tabs[k]);
             bpar.push_back(&it.p);
-            bsums.push_back(reinterpret_cast<double *>(wk + L.sums[k]));
             bout.push_back(it.out_dev);
         }
         if (bb.n)
-            PK_CUDA(launch_bin_batch(bb, btabs.data(), bpar.data(), bsums.data(), bout.data(), ctx->num_sms, st,
-                                     ctx->st),
+            PK_CUDA(launch_bin_batch(bb, btabs.data(), bpar.data(), bout.data(), ctx->num_sms, st, ctx->st),
                     "batched binning");
     }
     return PKMOM_OK;

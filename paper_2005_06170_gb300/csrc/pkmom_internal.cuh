@@ -65,9 +65,10 @@ struct AssignPlan {
     int64_t nkeys = 0;       // ng * ng * (ng >> sshift)
     int tile = 0;            // deposit tile id (see deposit launcher)
     int list_cap = 0;        // shared-memory particle list of an FP32 deposit tile (0 = none)
-    int hist_blocks = 0;     // blocks of the moments+histogram kernel
+    bool sparse = true;      // few particles per cell: orders 1 to 3 list their tiles too
+    int hist_blocks = 0;     // blocks of the histogram and scatter kernels
     int64_t scan_blocks = 0; // blocks of the key scan
-    size_t off_counts = 0, off_records = 0, off_partials = 0, off_blocksums = 0, off_qmax = 0;
+    size_t off_counts = 0, off_control = 0, off_records = 0, off_partials = 0, off_blocksums = 0;
     size_t off_halo = 0;     // home-tile deposit: per-tile halo nodes (0 = not used)
     size_t total = 0;
 };
@@ -85,7 +86,7 @@ struct FxJob {
     float *grids;
     int64_t grid_elems;
     long long first_tile;
-    int ng, sshift, list_cap, pad;
+    int ng, sshift, list_cap, sparse;
 };
 // The jobs of one launch, passed by value as the kernel's parameter (under 8 KB).
 constexpr int kBatchMax = 128;
@@ -115,13 +116,11 @@ struct BinBatch {
 };
 
 // ---------------------------------------------------------------- assign.cu
-cudaError_t launch_hist_moments(const pkmom_catalog &cat, const AssignPlan &pl, double box_L, void *scratch,
-                                int *err_flag, cudaStream_t s, LaunchStats &st);
-cudaError_t launch_moments_final(const AssignPlan &pl, int64_t n, void *scratch, double *moments_dev,
-                                 cudaStream_t s, LaunchStats &st);
+cudaError_t launch_hist(const pkmom_catalog &cat, const AssignPlan &pl, double box_L, void *scratch, int *err_flag,
+                        cudaStream_t s, LaunchStats &st);
 cudaError_t launch_scan(const AssignPlan &pl, void *scratch, cudaStream_t s, LaunchStats &st);
 cudaError_t launch_scatter(const pkmom_catalog &cat, const AssignPlan &pl, double box_L, void *scratch,
-                           cudaStream_t s, LaunchStats &st);
+                           double *moments_dev, cudaStream_t s, LaunchStats &st);
 cudaError_t launch_deposit(const AssignPlan &pl, void *scratch, void *grids, cudaStream_t s, LaunchStats &st);
 // Whether launch_deposit_batch can take this assignment (16^3 gather tiles, cubic, FP32,
 // exact BL kernel), and its FxJob (scratch and grids of that catalogue).
@@ -132,6 +131,8 @@ cudaError_t launch_deposit_batch(FxBatch &batch, unsigned long long *counter, in
                                  LaunchStats &st);
 // bytes of the key table (counts, then offsets) for nkeys sort keys
 size_t key_table_bytes(int64_t nkeys);
+// bytes of the control words zeroed with it
+size_t control_bytes();
 // Tile shapes the deposit kernel is instantiated for (x, y, z nodes).
 // Tile kHomeTile (16^3, FP32) deposits each particle once in the tile owning its cell
 // (cubic order; it needs home_halo_bytes of scratch); other orders use the 16^3 gather.
@@ -175,15 +176,16 @@ cudaError_t launch_bin_shells(const SpectraTables &t, const void *grids, const d
                               LaunchStats &st);
 // Persistent binning over the non-empty (slab, shell) items of many FP32 catalogues, each
 // into its own partials (ng * nbins * kBinVals doubles), then per catalogue the
-// fixed-order reduction into sums[kBinVals * nbins] (sums_of[k]) and the finalisation
-// into out[k]. batch.counter: 4 bytes of device memory the call zeroes and uses.
+// fixed-order reduction and finalisation into out[k]. batch.counter: 4 bytes of device
+// memory the call zeroes and uses.
 cudaError_t launch_bin_batch(BinBatch &batch, const SpectraTables *const *tables, const pkmom_params *const *params,
-                             double *const *sums_of, double *const *out, int num_sms, cudaStream_t s,
-                             LaunchStats &st);
-// sums_ready: the shell sums were already reduced (by launch_bin_shells); otherwise the
-// per-block partials of launch_bin are reduced first
+                             double *const *out, int num_sms, cudaStream_t s, LaunchStats &st);
+// The item partials of launch_bin_shells reduced per shell and turned into the output rows.
 cudaError_t launch_finalize(const SpectraTables &t, const pkmom_params &p, const double *moments_dev,
-                            double *out, cudaStream_t s, LaunchStats &st, bool sums_ready);
+                            double *out, cudaStream_t s, LaunchStats &st);
+// The same from the per-block partials of launch_bin.
+cudaError_t launch_finalize_blocks(const SpectraTables &t, const pkmom_params &p, const double *moments_dev,
+                                   double *out, cudaStream_t s, LaunchStats &st);
 
 // (|k|, mu)-binned spectra: per-item partials (ng * nbins * nmu items) and cell sums
 cudaError_t launch_spectra_mu(const SpectraTables &t, const pkmom_params &p, const void *grids,

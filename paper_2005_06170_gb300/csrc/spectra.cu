@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "pkmom_internal.cuh"
+#include "warp_sums.cuh"
 
 namespace pkmom {
 
@@ -165,54 +166,6 @@ k_bin(const Cx<T> *__restrict__ F, int64_t gstride, int ng, uint32_t nmodes, con
     __syncthreads();
     double *out = partials + static_cast<int64_t>(blockIdx.x) * kBinVals * nbins;
     for (int k = threadIdx.x; k < kBinVals * nbins; k += blockDim.x) out[k] = s_bins[k];
-}
-
-// (hi, lo) += (bh, bl) for unevaluated float pairs: a two-sum of the high parts, then
-// the low parts and the rounding error added and renormalised.
-__device__ __forceinline__ void pair_add(float &hi, float &lo, float bh, float bl)
-{
-    const float sh = __fadd_rn(hi, bh);
-    const float bb = __fsub_rn(sh, hi);
-    const float se = __fadd_rn(__fsub_rn(hi, __fsub_rn(sh, bb)), __fsub_rn(bh, bb));
-    const float t = __fadd_rn(se, __fadd_rn(lo, bl));
-    hi = __fadd_rn(sh, t);
-    lo = __fsub_rn(t, __fsub_rn(hi, sh));
-}
-__device__ __forceinline__ void pair_add(double &hi, double &lo, double bh, double bl)
-{
-    hi = (hi + lo) + (bh + bl);  // FP64: plain adds
-    lo = 0.0;
-}
-
-// Warp sums of 8 values per lane (value k as the pair hi[k] + lo[k]) by reduce-scatter:
-// at the steps across lanes 16, 8 and 4 apart each lane keeps half of the values it
-// still holds and adds its partner's copy of them, then the lanes 2 and 1 apart add their
-// single values. Lane L ends with the sum of value ((L >> 2) & 7) over the warp, the
-// same in lanes 4k..4k+3; 9 pair additions per lane instead of 40 for eight butterflies.
-// Returned as FP64; fixed order.
-template <typename T>
-__device__ __forceinline__ double warp_scatter_sum8(T (&hi)[8], T (&lo)[8])
-{
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int half = 4, o = 16; half >= 1; half >>= 1, o >>= 1) {
-        const bool up = (lane & o) != 0;  // keeps the upper half of its values
-#pragma unroll
-        for (int j = 0; j < half; ++j) {
-            const T mh = up ? hi[j + half] : hi[j], ml = up ? lo[j + half] : lo[j];
-            const T sh = up ? hi[j] : hi[j + half], sl = up ? lo[j] : lo[j + half];
-            const T rh = __shfl_xor_sync(full, sh, o), rl = __shfl_xor_sync(full, sl, o);
-            hi[j] = mh, lo[j] = ml;
-            pair_add(hi[j], lo[j], rh, rl);
-        }
-    }
-#pragma unroll
-    for (int o = 2; o >= 1; o >>= 1) {
-        const T rh = __shfl_xor_sync(full, hi[0], o), rl = __shfl_xor_sync(full, lo[0], o);
-        pair_add(hi[0], lo[0], rh, rl);
-    }
-    return static_cast<double>(hi[0]) + static_cast<double>(lo[0]);
 }
 
 // floor(sqrt(x)) for 0 <= x < 2^24, exact
@@ -394,9 +347,13 @@ k_bin_shells(const Cx<T> *__restrict__ F, int64_t gstride, int ng, int nbins, co
 {
     constexpr int NW = kBinThreads / 32;
     __shared__ BinWarpStage s_st[NW];
-    const double Mtot = mom[0];
-    const T vb0 = static_cast<T>(mom[2] / Mtot), vb1 = static_cast<T>(mom[3] / Mtot), vb2 = static_cast<T>(mom[4] / Mtot);
+    // v_b = sum m v / M by three lanes of the block: FP64 runs at under two lanes a clock per
+    // SM on this part, and the three divisions in every warp took 12 us of a launch
+    __shared__ T s_vb[3];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x < 3) s_vb[threadIdx.x] = static_cast<T>(mom[2 + threadIdx.x] / mom[0]);
+    __syncthreads();
+    const T vb0 = s_vb[0], vb1 = s_vb[1], vb2 = s_vb[2];
     for (;;) {
         unsigned j = 0;
         if (lane == 0) j = atomicAdd(counter, 1u);
@@ -417,7 +374,13 @@ k_bin_batch(const BinBatch jobs)
 {
     constexpr int NW = kBinThreads / 32;
     __shared__ BinWarpStage s_st[NW];
+    __shared__ float s_vb[3 * kBatchMax];  // v_b of every catalogue (see k_bin_shells)
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int k = threadIdx.x; k < 3 * jobs.n; k += kBinThreads) {
+        const double *mom = jobs.job[k / 3].mom;
+        s_vb[k] = static_cast<float>(mom[2 + k % 3] / mom[0]);
+    }
+    __syncthreads();
     int jj = 0;
     for (;;) {
         unsigned nx = 0;
@@ -426,9 +389,7 @@ k_bin_batch(const BinBatch jobs)
         if (item >= jobs.total_items) break;
         while (jj + 1 < jobs.n && jobs.job[jj + 1].first_item <= item) ++jj;  // items only grow
         const BinJob &jb = jobs.job[jj];
-        const double Mtot = jb.mom[0];
-        const float vb0 = static_cast<float>(jb.mom[2] / Mtot), vb1 = static_cast<float>(jb.mom[3] / Mtot),
-                    vb2 = static_cast<float>(jb.mom[4] / Mtot);
+        const float vb0 = s_vb[3 * jj], vb1 = s_vb[3 * jj + 1], vb2 = s_vb[3 * jj + 2];
         const int nh = jb.ng / 2 + 1;
         const int64_t gstride = static_cast<int64_t>(jb.ng) * jb.ng * nh;
         bin_item<float>(static_cast<const Cx<float> *>(jb.grids), gstride, jb.ng, jb.nbins, jb.thresh, jb.gf, jb.gh,
@@ -550,6 +511,78 @@ struct FinalParams {
 __device__ __forceinline__ double qdot(const double *Q, const double *H)
 {
     return Q[0] * H[0] + Q[1] * H[1] + Q[2] * H[2] + 2.0 * (Q[3] * H[3] + Q[4] * H[4] + Q[5] * H[5]);
+}
+
+// The item sums of a shell added over its slabs and turned into the output rows: one block
+// per shell, in a fixed order. FP64 runs at under two lanes a clock per SM here, so the
+// additions of a warp are a reduce-scatter and the rows are computed by lanes side by side:
+// lane r < 7 subtracts the shot noise of data row r (the same algebra as k_finalize). As two
+// kernels (item sums, then one thread a shell for all rows) the pair took 15 us, this 5.
+constexpr int kReduceThreads = 128;
+__global__ void __launch_bounds__(kReduceThreads)
+k_reduce_finalize(const double *__restrict__ partials, int nslabs, const int *__restrict__ thresh,
+                  const double *__restrict__ modes /*[kModeVals][nbins]*/, const double *__restrict__ mom,
+                  FinalParams fp, double *__restrict__ out)
+{
+    static_assert(kBinVals == 7, "rows of the seven data sums");
+    constexpr int NW = kReduceThreads / 32;
+    __shared__ double s_sum[NW][8];
+    const int b = blockIdx.x, nb = fp.nbins, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int hi2 = thresh[b + 1], lo2 = thresh[b];
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = 0.0;
+    for (int j = threadIdx.x; j < nslabs; j += kReduceThreads) {
+        const int n0 = j < nslabs / 2 ? j : j - nslabs;
+        if (hi2 <= lo2 || hi2 - 1 - n0 * n0 < 0) continue;  // the shell misses the slab: never written
+        const double *p = partials + (static_cast<int64_t>(j) * nb + b) * kBinVals;
+#pragma unroll
+        for (int k = 0; k < kBinVals; ++k) v[k] += p[k];
+    }
+    const double part = warp_scatter_sum8(v);
+    if ((lane & 3) == 0) s_sum[warp][lane >> 2] = part;
+    __syncthreads();
+    if (warp != 0) return;
+    const double n = modes[b];
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    if (!(n > 0.0)) {
+        if (lane < PKMOM_NROWS) out[lane * nb + b] = lane == PKMOM_ROW_NMODES ? n : nan;
+        return;
+    }
+    const int r = lane < 7 ? lane : 0;  // data row: dd, pp, tt, dt, pp', tt', dt'
+    double S = s_sum[0][r];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) S += s_sum[w][r];
+    const bool prime = r >= 4;
+    const double M = mom[0], S2 = mom[1];
+    const double *Q = mom + 8;
+    const int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};
+    double vb[3], Qr[6], H2[6];
+    for (int k = 0; k < 3; ++k) vb[k] = prime ? mom[2 + k] / M : 0.0;
+    // Q' = sum m^2 (v - v_b)(v - v_b)^T = Q - v_b R^T - R v_b^T + v_b v_b^T S2 (Sec. 3.1)
+    for (int k = 0; k < 6; ++k)
+        Qr[k] = Q[k] - vb[ia[k]] * mom[5 + ib[k]] - mom[5 + ia[k]] * vb[ib[k]] + vb[ia[k]] * vb[ib[k]] * S2;
+    for (int k = 0; k < 6; ++k) H2[k] = modes[(3 + k) * nb + b];
+    const double H = modes[2 * nb + b];
+    const double c = fp.V / (M * M * n);
+    const double ct = c * fp.ts * fp.ts * fp.kf * fp.kf, cx = c * fp.ts * fp.kf;
+    const double trQ = Qr[0] + Qr[1] + Qr[2], trH2 = H2[0] + H2[1] + H2[2];
+    const double sn_pp = c * trQ * H, sn_tt = ct * (fp.iso ? trQ * trH2 / 3.0 : qdot(Qr, H2));
+    const int kind = r == 0 ? 0 : (r - 1) % 3 + 1;  // dd, pp, tt, dt
+    const double sn = kind == 0 ? c * S2 * H : kind == 1 ? sn_pp : kind == 2 ? sn_tt : 0.0;
+    const double value = (kind == 2 ? ct : kind == 3 ? cx : c) * S - (fp.sub ? sn : 0.0);
+    if (lane < 7) {
+        const int rows[7] = {PKMOM_ROW_PDD,   PKMOM_ROW_PPP,   PKMOM_ROW_PTT,  PKMOM_ROW_PDT,
+                             PKMOM_ROW_PPP_B, PKMOM_ROW_PTT_B, PKMOM_ROW_PDT_B};
+        const int sn_rows[7] = {PKMOM_ROW_SNDD, PKMOM_ROW_SNPP, PKMOM_ROW_SNTT, -1, PKMOM_ROW_SNPP_B, PKMOM_ROW_SNTT_B, -1};
+        const bool absent = prime && !fp.bulk;
+        out[rows[r] * nb + b] = absent ? nan : value;
+        if (sn_rows[r] >= 0) out[sn_rows[r] * nb + b] = absent ? nan : sn;
+    } else if (lane == 7) {
+        out[PKMOM_ROW_K * nb + b] = fp.kf * modes[nb + b] / n;
+    } else if (lane == 8) {
+        out[PKMOM_ROW_NMODES * nb + b] = n;
+    }
 }
 
 __global__ void k_finalize(const double *__restrict__ sums /*[kBinVals][nbins]*/,
@@ -810,16 +843,12 @@ cudaError_t launch_bin_shells(const SpectraTables &t, const void *grids, const d
             static_cast<const Cx<double> *>(grids), gstride, ng, t.nbins, t.thresh,
             static_cast<const double *>(t.g_full), static_cast<const double *>(t.g_half), moments_dev, t.bin_order,
             t.bin_nwork, t.bin_counter, t.item_partials);
-    double *sums = t.mode_sums + static_cast<size_t>(kModeVals) * t.nbins;
-    k_reduce_items<kBinVals><<<t.nbins, 256, 0, s>>>(t.item_partials, ng, t.nbins, sums, t.thresh);
-    st.launches += 2;
+    st.launches++;
     return cudaGetLastError();
 }
 
 namespace {
-// k_finalize of shell sums `sums` ([kBinVals][nbins]) with the table's mode sums.
-cudaError_t finalize_sums(const SpectraTables &t, const pkmom_params &p, const double *moments_dev,
-                          const double *sums, double *out, cudaStream_t s, LaunchStats &st)
+FinalParams final_params(const SpectraTables &t, const pkmom_params &p)
 {
     FinalParams fp;
     fp.V = p.box_L * p.box_L * p.box_L;
@@ -829,14 +858,12 @@ cudaError_t finalize_sums(const SpectraTables &t, const pkmom_params &p, const d
     fp.bulk = p.bulk;
     fp.iso = p.theta_sn_mode == 1;
     fp.nbins = t.nbins;
-    k_finalize<<<(t.nbins + 127) / 128, 128, 0, s>>>(sums, t.mode_sums, moments_dev, fp, out);
-    st.launches++;
-    return cudaGetLastError();
+    return fp;
 }
 }  // namespace
 
 cudaError_t launch_bin_batch(BinBatch &batch, const SpectraTables *const *tables, const pkmom_params *const *params,
-                             double *const *sums_of, double *const *out, int num_sms, cudaStream_t s,
+                             double *const *out, int num_sms, cudaStream_t s,
                              LaunchStats &st)
 {
     long long first = 0;
@@ -858,31 +885,30 @@ cudaError_t launch_bin_batch(BinBatch &batch, const SpectraTables *const *tables
     }
     for (int k = 0; k < batch.n; ++k) {
         const BinJob &jb = batch.job[k];
-        k_reduce_items<kBinVals><<<jb.nbins, 256, 0, s>>>(jb.partials, jb.ng, jb.nbins, sums_of[k], jb.thresh);
+        k_reduce_finalize<<<jb.nbins, kReduceThreads, 0, s>>>(jb.partials, jb.ng, jb.thresh, tables[k]->mode_sums,
+                                                              jb.mom, final_params(*tables[k], *params[k]), out[k]);
         st.launches++;
-        if ((e = finalize_sums(*tables[k], *params[k], jb.mom, sums_of[k], out[k], s, st)) != cudaSuccess) return e;
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
 cudaError_t launch_finalize(const SpectraTables &t, const pkmom_params &p, const double *moments_dev, double *out,
-                            cudaStream_t s, LaunchStats &st, bool sums_ready)
+                            cudaStream_t s, LaunchStats &st)
+{
+    k_reduce_finalize<<<t.nbins, kReduceThreads, 0, s>>>(t.item_partials, t.ng, t.thresh, t.mode_sums, moments_dev,
+                                                         final_params(t, p), out);
+    st.launches++;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_finalize_blocks(const SpectraTables &t, const pkmom_params &p, const double *moments_dev,
+                                   double *out, cudaStream_t s, LaunchStats &st)
 {
     double *sums = t.mode_sums + static_cast<size_t>(kModeVals) * t.nbins;
-    if (!sums_ready) {
-        k_reduce_partials<kBinVals><<<t.nbins, 256, 0, s>>>(t.partials, t.bin_blocks, t.nbins, sums);
-        st.launches++;
-    }
-    FinalParams fp;
-    fp.V = p.box_L * p.box_L * p.box_L;
-    fp.kf = kTwoPi / p.box_L;
-    fp.ts = p.theta_scale;
-    fp.sub = p.subtract_shot_noise;
-    fp.bulk = p.bulk;
-    fp.iso = p.theta_sn_mode == 1;
-    fp.nbins = t.nbins;
-    k_finalize<<<(t.nbins + 127) / 128, 128, 0, s>>>(sums, t.mode_sums, moments_dev, fp, out);
-    st.launches++;
+    k_reduce_partials<kBinVals><<<t.nbins, 256, 0, s>>>(t.partials, t.bin_blocks, t.nbins, sums);
+    k_finalize<<<(t.nbins + 127) / 128, 128, 0, s>>>(sums, t.mode_sums, moments_dev, final_params(t, p), out);
+    st.launches += 2;
     return cudaGetLastError();
 }
 
@@ -1084,7 +1110,7 @@ extern "C" pkmom_status pkmom_spectra_static(const pkmom_params *p, const void *
     LaunchStats st;
     if (cudaGetLastError() != cudaSuccess) return PKMOM_ECUDA;
     if (launch_bin(t, grids, static_cast<const double *>(moments_dev), s, st) != cudaSuccess) return PKMOM_ECUDA;
-    if (launch_finalize(t, *p, static_cast<const double *>(moments_dev), out_dev, s, st, false) != cudaSuccess)
+    if (launch_finalize_blocks(t, *p, static_cast<const double *>(moments_dev), out_dev, s, st) != cudaSuccess)
         return PKMOM_ECUDA;
     return PKMOM_OK;
 }
