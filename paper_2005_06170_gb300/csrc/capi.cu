@@ -185,13 +185,16 @@ AssignPlan plan_assign(const pkmom_params &p, int64_t n, int num_sms, int tile_o
         ++sshift;
     pl.sshift = sshift;
     if (pl.tile == kHomeTile && sshift != 0) pl.tile = 0;  // home tiles need one sort key per cell
-    // sparse catalogues: list each tile's particles in shared memory (room for about
-    // twice the expected count of its reach; larger tiles fall back to searching)
+    // FP32 gather tiles list their particles in shared memory: room for about twice the
+    // expected count of a tile's reach, at most 2048 (longer ones go 2048 at a time).
+    // Orders 1 to 3 list sparse catalogues only: from half a particle per cell on, adding
+    // node by node was faster (TSC, 5 M particles on 200^3: 0.40 against 0.42 ms)
     const double reach = double(td[0] + 3) * (td[1] + 3) * (td[2] + 3);
-    if (p.precision == PKMOM_F32 && ppc < 0.5) {
+    if (p.precision == PKMOM_F32 && (ppc < 0.5 || p.order >= 4)) {
         const double want = 2.0 * ppc * reach + 64.0;
-        pl.list_cap = static_cast<int>(std::min(8192.0, std::ceil(want / 256.0) * 256.0));
+        pl.list_cap = static_cast<int>(std::min(2048.0, std::ceil(want / 256.0) * 256.0));
     }
+    pl.sparse = ppc < 0.5 || list_override >= 0;
     if (p.precision == PKMOM_F32 && list_override >= 0) pl.list_cap = std::min(list_override, 8192) / 32 * 32;
     pl.nkeys = int64_t(p.ng) * p.ng * (p.ng >> sshift);
     pl.hist_blocks = num_sms * 8;
