@@ -865,13 +865,14 @@ __device__ __forceinline__ void cell_chunk(const Record<float> *__restrict__ rec
     };
     uint32_t i = i0;
     for (; i + 4 <= i1; i += 4) {  // four loads in flight
-        const Record<float> r0 = rec[i], r1 = rec[i + 1], r2 = rec[i + 2], r3 = rec[i + 3];
+        const Record<float> r0 = load_record(rec + i), r1 = load_record(rec + i + 1), r2 = load_record(rec + i + 2),
+                            r3 = load_record(rec + i + 3);
         add(r0);
         add(r1);
         add(r2);
         add(r3);
     }
-    for (; i < i1; ++i) add(rec[i]);
+    for (; i < i1; ++i) add(load_record(rec + i));
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
         a[f] = round_shift(sa[f], shift[F0 + f]);
@@ -1668,14 +1669,17 @@ k_deposit_fx_batch(const FxBatch jobs, unsigned long long *__restrict__ counter)
 // each neighbour's halo to the owned nodes it overlaps, in a fixed order (so the grids
 // do not depend on scheduling).
 //
-// Lane mapping: a warp takes a block of 2 x 4 cell columns; lane (x, y, m) takes the
-// first particles of cells z = 4m .. 4m + 3 of its column and sums their contributions
-// to each node column's 7 z nodes in registers before adding them (home_quad), two
+// Lane mapping: a warp takes a block of 2 x 2 cell columns; lane (x, y, m) takes the
+// first particles of cells z = 2m, 2m + 1 of its column and sums their contributions
+// to each node column's 5 z nodes in registers before adding them (home_pair), two
 // fields' roundings per paired FMA (fma.rn.f32x2, each half the scalar FMA's result). The
 // buffer's x pitch is 16 modulo 32 banks, its y pitch 19 and its z pitch 1, so the 32
 // lanes of every add hit 32 different banks (checked at compile time below): one
 // wavefront each. Particles beyond the first of a cell go to a per-warp queue and are
-// deposited 32 at a time, one per lane.
+// deposited 32 at a time, one per lane. Bound by the shared pipe and by latency together
+// (shared memory holds two tiles per SM). Two cells a lane instead of four add 5 node sums
+// for 2 cells instead of 7 for 4, but fit 80 registers instead of 128, so that 24 warps run
+// on an SM instead of 16: 512^3 particles on 512^3, deposit 8.99 -> 8.75 ms.
 // Tiles with more than two particles per cell, or 32 in some four consecutive cells of a
 // column, take the cell-block path: one warp per cell, each contribution rounded at the
 // fine scale (largest contribution < 2^22) and summed exactly, in 64-bit shared
@@ -1692,33 +1696,35 @@ constexpr int kHomePY = kHomeB;                                 // buffer y pitc
 constexpr int kHomePX = 368;                                    // buffer x pitch
 constexpr int kHomeField = kHomeB * kHomePX;                    // ints per field
 constexpr int kHomeHalo = kHomeB * kHomeB * kHomeB - kHomeT * kHomeT * kHomeT;  // 2763 halo nodes
-constexpr int kHomeNT = 256;                                    // one thread per cell column of the tile
+constexpr int kHomeNT = 384;                                    // threads (at least one per cell column)
+constexpr int kHomeCP = 2;                                      // z-consecutive cells per lane
+constexpr int kHomeM = kHomeT / kHomeCP;                        // lanes per cell column
+constexpr int kHomeCols = 32 / kHomeM;                          // cell columns per warp step (2 in x)
+constexpr int kHomeColY = kHomeCols / 2;
 constexpr int kHomeNW = kHomeNT / 32;
 constexpr int kHomeQ = 64;                                      // overflow queue entries per warp
 constexpr size_t kHomeSmem = size_t(4) * kHomeField * sizeof(int);
 static_assert(kHomePX % 32 == 16 && kHomePX >= kHomeB * kHomeB, "x-adjacent cells must be 16 banks apart");
-static_assert(kHomeNT == kHomeT * kHomeT, "one thread per cell column");
-static_assert(kHomeNW * kHomeQ <= 2 * kHomeNT + 1, "queues share the column-range arrays");
+static_assert(kHomeNT >= kHomeT * kHomeT, "one thread per cell column");
 
-// Banks of the first stencil node of the 32 lanes of a four-cells-per-lane block (2 x 4
-// columns, lane (x, y, m) at cells z = 4m .. 4m + 3): all different, so that every add
-// of home_quad is one wavefront.
-constexpr bool home_quad_banks_distinct()
+// Banks of the first stencil node of the 32 lanes of a block (2 x 2 columns, lane (x, y, m)
+// at cells z = 2m, 2m + 1): all different, so that every add of home_pair is one wavefront.
+constexpr bool home_pair_banks_distinct()
 {
     unsigned seen = 0;
     for (int lane = 0; lane < 32; ++lane) {
-        const int m = lane & 3, y = (lane >> 2) & 3, x = lane >> 4;
-        const unsigned bit = 1u << ((x * kHomePX + y * kHomePY + 4 * m) & 31);
+        const int m = lane % kHomeM, y = (lane / kHomeM) % kHomeColY, x = lane / (kHomeM * kHomeColY);
+        const unsigned bit = 1u << ((x * kHomePX + y * kHomePY + kHomeCP * m) & 31);
         if (seen & bit) return false;
         seen |= bit;
     }
     return true;
 }
-static_assert(home_quad_banks_distinct(), "the 32 lanes of a home_quad add must hit 32 banks");
-// home_quad's largest buffer index on each axis: cell 15 + node offset 3 in x and y,
-// z = 4 * 3 + 6 (seven z nodes from the lane's first cell); all inside the 19-node edge
-static_assert(kHomeT - 1 + 3 < kHomeB && 4 * 3 + 6 < kHomeB && kHomeT % 4 == 0 && kHomeT / 4 == 4,
-              "home_quad's nodes must lie in the node buffer");
+static_assert(home_pair_banks_distinct(), "the 32 lanes of a home_pair add must hit 32 banks");
+// home_pair's largest buffer index on each axis: cell 15 + node offset 3 in x and y, and
+// CP + 3 z nodes from the lane's first cell; all inside the 19-node edge
+static_assert(kHomeT - 1 + 3 < kHomeB && kHomeT - kHomeCP + kHomeCP + 2 < kHomeB && kHomeT % kHomeCP == 0,
+              "home_pair's nodes must lie in the node buffer");
 
 // Halo index of buffer node (bx, by, bz), at least one coordinate in {0, 17, 18}:
 // first the three x planes (19 x 19 each), then the y planes of the inner x range
@@ -1826,9 +1832,10 @@ __device__ __forceinline__ void home_pair(unsigned acc_s, const Record<float> (&
 {
     constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
     constexpr unsigned kMagicBits = 0x4B400000u;
-    float wx[4][4], wy[4][4], wz[4][4], q[4][4];
+    constexpr int CP = kHomeCP;
+    float wx[CP][4], wy[CP][4], wz[CP][4], q[CP][4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < CP; ++j) {
         int first;
         bspline_weights<4, float>(has[j] ? r[j].u.x : 0.0f, wx[j], first);
         bspline_weights<4, float>(has[j] ? r[j].u.y : 0.0f, wy[j], first);
@@ -1838,29 +1845,29 @@ __device__ __forceinline__ void home_pair(unsigned acc_s, const Record<float> (&
         q[j][2] = has[j] ? r[j].q.z * sc2 : 0.0f;
         q[j][3] = has[j] ? r[j].q.w * sc3 : 0.0f;
     }
-    f32x2 qp[4][2];  // fields (0, 1) and (2, 3) of each cell as pairs
+    f32x2 qp[CP][2];  // fields (0, 1) and (2, 3) of each cell as pairs
 #pragma unroll
-    for (int j = 0; j < 4; ++j) qp[j][0] = f2_pack(q[j][0], q[j][1]), qp[j][1] = f2_pack(q[j][2], q[j][3]);
+    for (int j = 0; j < CP; ++j) qp[j][0] = f2_pack(q[j][0], q[j][1]), qp[j][1] = f2_pack(q[j][2], q[j][3]);
     const f32x2 mg = f2_pack(kMagic, kMagic);
-    // buffer index of node (cx - 1 + dx, cy - 1 + dy, 4m - 1 + i) is (cx + dx) PX + (cy + dy) PY + 4m + i.
+    // buffer index of node (cx - 1 + dx, cy - 1 + dy, CP m - 1 + i) is (cx + dx) PX + (cy + dy) PY + CP m + i.
     // The 4 x 4 node columns are two rolled loops (a short body for the instruction
     // cache); the weights of the current dx and dy are kept in slot 0 by rotating them.
-    // the lane's last node (3, 3 node columns on, z node 4m + 6) must lie in the buffer
-    if (!PK_IN((cx + 3) * kHomePX + (cy + 3) * kHomePY + 4 * m + 6, kHomeField, kChkShared)) return;
-    unsigned base = acc_s + 4u * static_cast<unsigned>(cx * kHomePX + cy * kHomePY + 4 * m);
+    // the lane's last node (3, 3 node columns on) must lie in the buffer
+    if (!PK_IN((cx + 3) * kHomePX + (cy + 3) * kHomePY + CP * m + CP + 2, kHomeField, kChkShared)) return;
+    unsigned base = acc_s + 4u * static_cast<unsigned>(cx * kHomePX + cy * kHomePY + CP * m);
 #pragma unroll 1
     for (int dx = 0; dx < 4; ++dx) {
 #pragma unroll 1
         for (int dy = 0; dy < 4; ++dy) {
-            unsigned a[7][4];
-            static_for<7>([&](auto ic) {
+            unsigned a[CP + 3][4];
+            static_for<CP + 3>([&](auto ic) {
                 constexpr int i = decltype(ic)::value;
-                constexpr unsigned cnt = static_cast<unsigned>((i < 3 ? i : 3) - (i > 3 ? i - 3 : 0) + 1);
+                constexpr unsigned cnt = static_cast<unsigned>((i < CP - 1 ? i : CP - 1) - (i > 3 ? i - 3 : 0) + 1);
 #pragma unroll
                 for (int f = 0; f < 4; ++f) a[i][f] = 0u - cnt * kMagicBits;
             });
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < CP; ++j) {
                 const float w01 = wx[j][0] * wy[j][0];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
@@ -1874,19 +1881,19 @@ __device__ __forceinline__ void home_pair(unsigned acc_s, const Record<float> (&
                 }
             }
             const unsigned b = base + 4u * static_cast<unsigned>(dy * kHomePY);
-            static_for<7>([&](auto ic) {
+            static_for<CP + 3>([&](auto ic) {
                 constexpr int i = decltype(ic)::value;
                 red4<4 * i, 4 * kHomeField>(b, static_cast<int>(a[i][0]), static_cast<int>(a[i][1]),
                                             static_cast<int>(a[i][2]), static_cast<int>(a[i][3]));
             });
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {  // next dy in slot 0
+            for (int j = 0; j < CP; ++j) {  // next dy in slot 0
                 const float t = wy[j][0];
                 wy[j][0] = wy[j][1], wy[j][1] = wy[j][2], wy[j][2] = wy[j][3], wy[j][3] = t;
             }
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {  // next dx in slot 0
+        for (int j = 0; j < CP; ++j) {  // next dx in slot 0
             const float t = wx[j][0];
             wx[j][0] = wx[j][1], wx[j][1] = wx[j][2], wx[j][2] = wx[j][3], wx[j][3] = t;
         }
@@ -1899,7 +1906,7 @@ __device__ __forceinline__ void home_pair(unsigned acc_s, const Record<float> (&
 __device__ __noinline__ void home_listed(int *acc, const Record<float> *__restrict__ rec, uint32_t idx, int t0, int t1,
                                          int t2, float sc0, float sc1, float sc2, float sc3)
 {
-    const Record<float> r = rec[idx];
+    const Record<float> r = load_record(rec + idx);
     const int c = unpack_cell(r.u.w);
     const unsigned cx = static_cast<unsigned>((c & 1023) - t0), cy = static_cast<unsigned>(((c >> 10) & 1023) - t1),
                    cz = static_cast<unsigned>(((c >> 20) & 1023) - t2);
@@ -1907,37 +1914,64 @@ __device__ __noinline__ void home_listed(int *acc, const Record<float> *__restri
         home_particle(acc, r, static_cast<int>(cx), static_cast<int>(cy), static_cast<int>(cz), sc0, sc1, sc2, sc3);
 }
 
-// Dense home tiles: one warp per occupied cell; lane l owns stencil nodes (dx, dy, dz)
-// with dz = l & 3, dy = (l >> 2) & 3, dx = (l >> 4) and (l >> 4) + 2, sums up to
-// kCellFlush of the cell's particles in FP32 registers and adds the rounded sums.
+// Dense home tiles: one warp per cell column; lane l owns stencil nodes (dx, dy, dz)
+// with dz = l & 3, dy = (l >> 2) & 3, dx = (l >> 4) and (l >> 4) + 2 of the cell at hand, sums
+// up to kCellFlush of the cell's particles in registers and adds the sums to 64-bit totals,
+// two fields per pass. limbs: the totals are kept as two 32-bit words, the low 16 bits of each
+// sum and the rest (a 64-bit shared add takes as long as eight 32-bit ones; a node gets fewer
+// than 2^16 sums, see the caller); otherwise as 64-bit words. The column's 17 offsets are
+// loaded at once and its records asked for ahead: cell by cell, the two dependent loads of
+// each of 4096 cells were most of the time.
 template <int F0>
 __device__ __forceinline__ void home_cells_path(const Record<float> *__restrict__ rec,
                                                 const uint32_t *__restrict__ offsets, int ng, int t0, int t1, int t2,
-                                                unsigned long long *acc, const float *s_fine)
+                                                unsigned char *acc, bool limbs, const float *s_fine)
 {
     const float fine[4] = {s_fine[0], s_fine[1], s_fine[2], s_fine[3]};
     const int noshift[4] = {0, 0, 0, 0};
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int dz = lane & 3, dy = (lane >> 2) & 3, dxl = lane >> 4;
+    auto *acc64 = reinterpret_cast<unsigned long long *>(acc);  // [2][kHomeField]
+    int *acc32 = reinterpret_cast<int *>(acc);                  // [2 fields][low, high][kHomeField]
     CellPieces pc;
     cubic_piece(dxl, pc.xa);
     cubic_piece(dxl + 2, pc.xb);
     cubic_piece(dy, pc.y);
     cubic_piece(dz, pc.z);
-    for (int c = warp; c < kHomeT * kHomeT * kHomeT; c += kHomeNW) {
-        const int cx = c >> 8, cy = (c >> 4) & 15, cz = c & 15;
-        const int64_t key = (static_cast<int64_t>(t0 + cx) * ng + (t1 + cy)) * ng + (t2 + cz);
-        const uint32_t beg = offsets[key], end = offsets[key + 1];
-        if (beg == end) continue;
-        const int oa = (cx + dxl) * kHomePX + (cy + dy) * kHomePY + cz + dz, ob = oa + 2 * kHomePX;
-        if (!PK_IN(ob, kHomeField, kChkShared)) continue;
-        for (uint32_t i0 = beg; i0 < end; i0 += kCellFlush) {
-            int a[2], b[2];
-            cell_chunk<F0, 2>(rec, i0, min(end, i0 + kCellFlush), pc, fine, noshift, a, b);
+    auto column_offset = [&](int col) -> uint32_t {  // lane z: offset of cell z of the column
+        if (col >= kHomeT * kHomeT || lane > kHomeT) return 0u;
+        return offsets[(static_cast<int64_t>(t0 + (col >> 4)) * ng + (t1 + (col & 15))) * ng + t2 + lane];
+    };
+    uint32_t next = column_offset(warp);
+    for (int col = warp; col < kHomeT * kHomeT; col += kHomeNW) {
+        const uint32_t o = next;
+        next = column_offset(col + kHomeNW);
+        const uint32_t first = __shfl_sync(0xffffffffu, o, 0), last = __shfl_sync(0xffffffffu, o, kHomeT);
+        for (uint32_t i = first + 4 * lane; i < last && i < first + 512; i += 128)
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(rec + i));
+        const uint32_t after = __shfl_down_sync(0xffffffffu, o, 1);
+        for (unsigned full = __ballot_sync(0xffffffffu, lane < kHomeT && after > o); full; full &= full - 1u) {
+            const int cz = __ffs(static_cast<int>(full)) - 1;
+            const uint32_t beg = __shfl_sync(0xffffffffu, o, cz), end = __shfl_sync(0xffffffffu, after, cz);
+            const int oa = ((col >> 4) + dxl) * kHomePX + ((col & 15) + dy) * kHomePY + cz + dz, ob = oa + 2 * kHomePX;
+            if (!PK_IN(ob, kHomeField, kChkShared)) continue;
+            for (uint32_t i0 = beg; i0 < end; i0 += kCellFlush) {
+                int a[2], b[2];
+                cell_chunk<F0, 2>(rec, i0, min(end, i0 + kCellFlush), pc, fine, noshift, a, b);
 #pragma unroll
-            for (int f = 0; f < 2; ++f) {  // two's complement sums
-                atomicAdd(acc + f * kHomeField + oa, static_cast<unsigned long long>(static_cast<long long>(a[f])));
-                atomicAdd(acc + f * kHomeField + ob, static_cast<unsigned long long>(static_cast<long long>(b[f])));
+                for (int f = 0; f < 2; ++f) {  // two's complement sums
+                    if (limbs) {
+                        int *n = acc32 + 2 * f * kHomeField;
+                        atomicAdd(n + oa, a[f] & 0xffff);
+                        atomicAdd(n + kHomeField + oa, a[f] >> 16);
+                        atomicAdd(n + ob, b[f] & 0xffff);
+                        atomicAdd(n + kHomeField + ob, b[f] >> 16);
+                    } else {
+                        unsigned long long *n = acc64 + f * kHomeField;
+                        atomicAdd(n + oa, static_cast<unsigned long long>(static_cast<long long>(a[f])));
+                        atomicAdd(n + ob, static_cast<unsigned long long>(static_cast<long long>(b[f])));
+                    }
+                }
             }
         }
     }
@@ -1951,8 +1985,8 @@ k_deposit_home(const Record<float> *__restrict__ rec, const uint32_t *__restrict
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int *acc = reinterpret_cast<int *>(smem_raw);  // [4][kHomeB][kHomePX] (x, y, z of the node buffer)
     // column ranges of the tile (sparse path), reused as the per-warp queues (medium path)
-    __shared__ uint32_t s_cols[2 * kHomeNT + 1];
-    uint32_t *s_beg = s_cols, *s_pre = s_cols + kHomeNT;
+    __shared__ uint32_t s_cols[kHomeNW * kHomeQ > 2 * kHomeT * kHomeT + 1 ? kHomeNW * kHomeQ : 2 * kHomeT * kHomeT + 1];
+    uint32_t *s_beg = s_cols, *s_pre = s_cols + kHomeT * kHomeT;
     __shared__ unsigned s_rowmax;
     __shared__ float s_scale[4], s_fine[4];
     __shared__ int s_shift[4];
@@ -1970,12 +2004,17 @@ k_deposit_home(const Record<float> *__restrict__ rec, const uint32_t *__restrict
     // thread = cell column (x, y) of the tile: its particles are one range of the sort
     uint32_t total;
     {
-        const int x = threadIdx.x >> 4, y = threadIdx.x & 15;
+        const bool col = threadIdx.x < kHomeT * kHomeT;
+        const int x = (threadIdx.x >> 4) & 15, y = threadIdx.x & 15;
         const int64_t key = (static_cast<int64_t>(t0 + x) * ng + (t1 + y)) * ng + t2;
-        uint32_t o[kHomeT + 1];
+        uint32_t o[kHomeT + 1];  // offsets[key + 1] is 16-byte aligned (key_table), keys per column 16
+        o[0] = offsets[key];
 #pragma unroll
-        for (int z = 0; z <= kHomeT; ++z) o[z] = offsets[key + z];
-        const uint32_t b = o[0], cnt = o[kHomeT] - b;
+        for (int z = 0; z < kHomeT; z += 4) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(offsets + key + 1 + z);
+            o[z + 1] = v.x, o[z + 2] = v.y, o[z + 3] = v.z, o[z + 4] = v.w;
+        }
+        const uint32_t b = o[0], cnt = col ? o[kHomeT] - b : 0u;
         // the column's records are read later, cell by cell: ask L2 for them now (128-byte
         // lines covering the column's contiguous range, at most 32 lines per column)
         {
@@ -1988,9 +2027,8 @@ k_deposit_home(const Record<float> *__restrict__ rec, const uint32_t *__restrict
 #pragma unroll
         for (int z = 0; z + 4 <= kHomeT; ++z) win = max(win, o[z + 4] - o[z]);
         const uint32_t pre = block_exclusive_scan(cnt, total);
-        s_beg[threadIdx.x] = b;
-        s_pre[threadIdx.x] = pre;
-        if (threadIdx.x == 0) s_pre[kHomeNT] = total;
+        if (col) s_beg[threadIdx.x] = b, s_pre[threadIdx.x] = pre;
+        if (threadIdx.x == 0) s_pre[kHomeT * kHomeT] = total;
         if (win) atomicMax(&s_rowmax, win);
     }
     __syncthreads();
@@ -2019,8 +2057,8 @@ k_deposit_home(const Record<float> *__restrict__ rec, const uint32_t *__restrict
     auto emit = [&](int f, auto value) {
         float *gf = grids + f * grid_elems;
 #pragma unroll 2
-        for (int pass = 0; pass < kHomeT * kHomeT * 8 / kHomeNT; ++pass) {
-            const int rowi = pass * (kHomeNT / 8) + (threadIdx.x >> 3), zp = 2 * (threadIdx.x & 7);
+        for (int rowi = threadIdx.x >> 3; rowi < kHomeT * kHomeT; rowi += kHomeNT / 8) {
+            const int zp = 2 * (threadIdx.x & 7);
             const int x = rowi >> 4, y = rowi & 15;
             const int ab = (x + 1) * kHomePX + (y + 1) * kHomePY + zp + 1;
             const int64_t gi = (static_cast<int64_t>(t0 + x) * ng + (t1 + y)) * (ng + 2) + t2 + zp;
@@ -2039,8 +2077,11 @@ k_deposit_home(const Record<float> *__restrict__ rec, const uint32_t *__restrict
     };
 
     if (dense) {
-        // 64-bit sums of the fine-scale contributions, two fields per pass in the same buffer
-        auto *acc64 = reinterpret_cast<unsigned long long *>(smem_raw);  // [2][kHomeB][kHomePX]
+        // 64-bit sums of the fine-scale contributions, two fields per pass in the same buffer.
+        // A node gets one sum from each of 64 cells per kCellFlush particles: up to 2^23
+        // particles fewer than 2^16 sums, each below 2^30, so that the low words' sum stays
+        // below 2^32 and the high words' below 2^30
+        const bool limbs = total <= 1u << 23;
 #pragma unroll
         for (int pass = 0; pass < 2; ++pass) {
             if (pass) {
@@ -2049,15 +2090,21 @@ k_deposit_home(const Record<float> *__restrict__ rec, const uint32_t *__restrict
                 for (int k = threadIdx.x; k < kHomeField; k += kHomeNT) a4[k] = make_int4(0, 0, 0, 0);
                 __syncthreads();
             }
-            if (pass == 0) home_cells_path<0>(rec, offsets, ng, t0, t1, t2, acc64, s_fine);
-            else home_cells_path<2>(rec, offsets, ng, t0, t1, t2, acc64, s_fine);
+            if (pass == 0) home_cells_path<0>(rec, offsets, ng, t0, t1, t2, smem_raw, limbs, s_fine);
+            else home_cells_path<2>(rec, offsets, ng, t0, t1, t2, smem_raw, limbs, s_fine);
             __syncthreads();
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const int f = 2 * pass + k;
                 const float inv = 1.0f / s_fine[f];  // exact: a power of two
-                const unsigned long long *a = acc64 + k * kHomeField;
-                emit(f, [&](int ai) { return static_cast<float>(static_cast<long long>(a[ai])) * inv; });
+                const auto *a64 = reinterpret_cast<const long long *>(smem_raw) + k * kHomeField;
+                const int *a32 = acc + 2 * k * kHomeField;
+                emit(f, [&](int ai) {
+                    const long long v = limbs ? static_cast<long long>(a32[kHomeField + ai]) * 65536 +
+                                                    static_cast<unsigned>(a32[ai])
+                                              : a64[ai];
+                    return static_cast<float>(v) * inv;
+                });
             }
         }
         return;
@@ -2066,7 +2113,7 @@ k_deposit_home(const Record<float> *__restrict__ rec, const uint32_t *__restrict
         // one particle per lane, warp-contiguous chunks of the tile's list
         const uint32_t per_warp = ((total + kHomeNW - 1) / kHomeNW + 31u) & ~31u;
         const uint32_t wbeg = static_cast<uint32_t>(warp) * per_warp, wend = min(wbeg + per_warp, total);
-        int slot = wbeg + lane < wend ? find_slot<kHomeNT>(s_pre, wbeg + lane) : 0;
+        int slot = wbeg + lane < wend ? find_slot<kHomeT * kHomeT>(s_pre, wbeg + lane) : 0;
         for (uint32_t p = wbeg + lane; p < wend; p += 32) {
             while (p >= s_pre[slot + 1]) ++slot;
             home_listed(acc, rec, s_beg[slot] + (p - s_pre[slot]), t0, t1, t2, sc0, sc1, sc2, sc3);
@@ -2076,39 +2123,46 @@ k_deposit_home(const Record<float> *__restrict__ rec, const uint32_t *__restrict
         __syncthreads();
         int qn = 0;  // warp-uniform queue length
         const unsigned acc_s = static_cast<unsigned>(__cvta_generic_to_shared(acc));
-        // a block is 2 x 4 cell columns; lane (xl, yl, m) takes cells z = 4m .. 4m + 3
-        const int m = lane & 3, yl = (lane >> 2) & 3, xl = lane >> 4;
-        constexpr int kBlocks = (kHomeT / 2) * (kHomeT / 4);
-        auto cell_offsets = [&](int blk, uint32_t(&o)[5]) {  // the five offsets of the four cells
+        // a block is 2 x kHomeColY cell columns; lane (xl, yl, m) takes the kHomeCP cells from z = kHomeCP m
+        constexpr int CP = kHomeCP, BY = kHomeT / kHomeColY;
+        const int m = lane % kHomeM, yl = (lane / kHomeM) % kHomeColY, xl = lane / (kHomeM * kHomeColY);
+        constexpr int kBlocks = (kHomeT / 2) * BY;
+        auto cell_offsets = [&](int blk, uint32_t(&o)[CP + 1]) {  // the offsets of the lane's cells
             if (blk >= kBlocks) {
 #pragma unroll
-                for (int k = 0; k < 5; ++k) o[k] = 0;
+                for (int k = 0; k <= CP; ++k) o[k] = 0;
                 return;
             }
-            const int cx = 2 * (blk >> 2) + xl, cy = 4 * (blk & 3) + yl;
-            const int64_t key = (static_cast<int64_t>(t0 + cx) * ng + (t1 + cy)) * ng + (t2 + 4 * m);
-#pragma unroll
-            for (int k = 0; k < 5; ++k) o[k] = offsets[key + k];
+            const int cx = 2 * (blk / BY) + xl, cy = kHomeColY * (blk % BY) + yl;
+            const int64_t key = (static_cast<int64_t>(t0 + cx) * ng + (t1 + cy)) * ng + (t2 + CP * m);
+            o[0] = offsets[key];
+            if constexpr (CP == 4) {
+                const uint4 v = *reinterpret_cast<const uint4 *>(offsets + key + 1);
+                o[1] = v.x, o[2] = v.y, o[CP - 1] = v.z, o[CP] = v.w;
+            } else {
+                const uint2 v = *reinterpret_cast<const uint2 *>(offsets + key + 1);
+                o[1] = v.x, o[2] = v.y;
+            }
         };
-        uint32_t on[5];
+        uint32_t on[CP + 1];
         cell_offsets(warp, on);  // loads run one block ahead
         for (int blk = warp; blk < kBlocks; blk += kHomeNW) {
-            const int cx = 2 * (blk >> 2) + xl, cy = 4 * (blk & 3) + yl;
-            uint32_t o[5];
+            const int cx = 2 * (blk / BY) + xl, cy = kHomeColY * (blk % BY) + yl;
+            uint32_t o[CP + 1];
 #pragma unroll
-            for (int k = 0; k < 5; ++k) o[k] = on[k];
+            for (int k = 0; k <= CP; ++k) o[k] = on[k];
             cell_offsets(blk + kHomeNW, on);
-            Record<float> r[4];
-            bool has[4];
+            Record<float> r[CP];
+            bool has[CP];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
+            for (int k = 0; k < CP; ++k) {
                 has[k] = o[k + 1] > o[k];
-                r[k] = has[k] ? rec[o[k]] : Record<float>{};
+                r[k] = has[k] ? load_record(rec + o[k]) : Record<float>{};
             }
-            home_quad(acc_s, r, has, cx, cy, m, sc0, sc1, sc2, sc3);
-            // second and later particles of the four cells: the per-warp queue, 32 at a time
+            home_pair(acc_s, r, has, cx, cy, m, sc0, sc1, sc2, sc3);
+            // second and later particles of the cells: the per-warp queue, 32 at a time
 #pragma unroll 1
-            for (int k = 0; k < 4; ++k) {
+            for (int k = 0; k < CP; ++k) {
                 uint32_t next = o[k] + 1, extra = has[k] ? o[k + 1] - o[k] - 1 : 0u;
                 while (__any_sync(0xffffffffu, extra > 0u)) {
                     const bool more = extra > 0u;
