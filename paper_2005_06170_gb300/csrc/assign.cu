@@ -128,8 +128,8 @@ __device__ __forceinline__ void static_for(F &&f)
 
 __device__ __forceinline__ int floordiv(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
-// A record's fourth coordinate holds its wrapped cell (10 bits per axis, ng <= 1024):
-// the bit pattern of an FP32 value, or the integer itself as an FP64 value.
+// A record's fourth coordinate holds its wrapped cell (10 bits per axis, ng <= 1024) as a
+// bit pattern.
 template <typename T> __device__ __forceinline__ T pack_cell(int c0, int c1, int c2);
 template <> __device__ __forceinline__ float pack_cell<float>(int c0, int c1, int c2)
 {
@@ -137,10 +137,10 @@ template <> __device__ __forceinline__ float pack_cell<float>(int c0, int c1, in
 }
 template <> __device__ __forceinline__ double pack_cell<double>(int c0, int c1, int c2)
 {
-    return static_cast<double>(c0 | (c1 << 10) | (c2 << 20));
+    return __longlong_as_double(c0 | (c1 << 10) | (c2 << 20));
 }
 __device__ __forceinline__ int unpack_cell(float v) { return __float_as_int(v); }
-__device__ __forceinline__ int unpack_cell(double v) { return static_cast<int>(v); }
+__device__ __forceinline__ int unpack_cell(double v) { return static_cast<int>(__double_as_longlong(v)); }
 
 // The histogram of sort keys: positions only (12 bytes per FP32 particle), one
 // fire-and-forget atomic increment per particle; non-finite or huge positions raise
@@ -294,13 +294,14 @@ template <typename T, bool MASS>
 struct LaneMoments {
     static constexpr int NV = MASS ? kMomentVals : 9;
     T sum[NV], cmp[NV];  // the sum of a value is sum - cmp
-    T qmax[4];
+    // FP32: max |q| of each field; FP64: the high words of the largest |q| (NaN above all)
+    std::conditional_t<sizeof(T) == 4, float, int> qmax[4];
     __device__ __forceinline__ LaneMoments()
     {
 #pragma unroll
         for (int k = 0; k < NV; ++k) sum[k] = T(0), cmp[k] = T(0);
 #pragma unroll
-        for (int f = 0; f < 4; ++f) qmax[f] = T(0);
+        for (int f = 0; f < 4; ++f) qmax[f] = 0;
     }
     __device__ __forceinline__ void put(int k, T x)
     {
@@ -348,7 +349,7 @@ struct LaneMoments {
     __device__ __forceinline__ void top(int f, T x)
     {
         if constexpr (sizeof(T) == 4) qmax[f] = fmaxf(qmax[f], fabsf(x));
-        else qmax[f] = fabs(x) > qmax[f] ? fabs(x) : qmax[f];
+        else qmax[f] = max(qmax[f], __double2hiint(x) & 0x7fffffff);
     }
 };
 
@@ -385,11 +386,15 @@ __device__ __forceinline__ void finish_moments(LaneMoments<T, MASS> &lm, int64_t
         }
         if ((lane & 3) == 0) s_part[warp][8 * g + (lane >> 2)] = x;
     }
-    if constexpr (!MASS) lm.qmax[0] = T(1);
+    if constexpr (!MASS && sizeof(T) == 4) lm.qmax[0] = 1.0f;
+    else if constexpr (!MASS) lm.qmax[0] = 0x3ff00000;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
         // non-negative floats order like their bit patterns
-        const unsigned bits = __reduce_max_sync(0xffffffffu, __float_as_uint(static_cast<float>(lm.qmax[f])));
+        unsigned mine;
+        if constexpr (sizeof(T) == 4) mine = __float_as_uint(lm.qmax[f]);
+        else mine = static_cast<unsigned>(lm.qmax[f]);
+        const unsigned bits = __reduce_max_sync(0xffffffffu, mine);
         if (lane == 0) atomicMax(qmax_bits + f, bits);
     }
     __syncthreads();
@@ -739,20 +744,15 @@ __device__ __forceinline__ bool bl_node_x(const Record<T> &r, int ng, int t0, in
     return true;
 }
 
-// Tile-gather deposit with shared-memory atomics in the grid precision (used for
-// FP64 grids, where FP64 accuracy is required).
-template <typename T, int M, int T0, int T1, int T2, int NT, int BLR = 0>
-__global__ void __launch_bounds__(NT)
-k_deposit(const Record<T> *__restrict__ rec, const uint32_t *__restrict__ offsets,
-          const unsigned *__restrict__ /*qmax_bits*/, int ng, int sshift, T *__restrict__ grids, int64_t grid_elems,
-          int /*list_cap*/, bool /*sparse*/)
+// FP64 tile-gather deposit with FP64 shared-memory atomics, for the cases the fixed-point
+// deposit (k_deposit_ix) leaves out. The whole CTA takes part; acc: 4 T0 T1 T2 words.
+template <typename T, int M, int T0, int T1, int T2, int NT, int BLR>
+__device__ __noinline__ void deposit_fp64_tile(const Record<T> *__restrict__ rec,
+                                               const uint32_t *__restrict__ offsets, int ng, int sshift,
+                                               T *__restrict__ grids, int64_t grid_elems, T *acc, uint32_t *s_beg,
+                                               uint32_t *s_pre)
 {
     using C = DepositCfg<T, M, T0, T1, T2, NT>;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *acc = reinterpret_cast<T *>(smem_raw);  // [4][T0][T1][T2]
-    __shared__ uint32_t s_beg[C::MAXR];
-    __shared__ uint32_t s_pre[C::MAXR + 1];
-
     const int ntz = ng / T2, nty = ng / T1;
     int tile = blockIdx.x;
     const int tz = tile % ntz;
@@ -807,6 +807,371 @@ k_deposit(const Record<T> *__restrict__ rec, const uint32_t *__restrict__ offset
         if (!PK_IN(gi, grid_elems, kChkGrid)) continue;
 #pragma unroll
         for (int f = 0; f < 4; ++f) grids[f * grid_elems + gi] = acc[f * C::TN + k];
+    }
+}
+
+template <typename T, int M, int T0, int T1, int T2, int NT, int BLR = 0>
+__global__ void __launch_bounds__(NT)
+k_deposit(const Record<T> *__restrict__ rec, const uint32_t *__restrict__ offsets,
+          const unsigned *__restrict__ /*qmax_bits*/, int ng, int sshift, T *__restrict__ grids, int64_t grid_elems,
+          int /*list_cap*/, bool /*sparse*/)
+{
+    using C = DepositCfg<T, M, T0, T1, T2, NT>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint32_t s_beg[C::MAXR];
+    __shared__ uint32_t s_pre[C::MAXR + 1];
+    deposit_fp64_tile<T, M, T0, T1, T2, NT, BLR>(rec, offsets, ng, sshift, grids, grid_elems,
+                                                 reinterpret_cast<T *>(smem_raw), s_beg, s_pre);
+}
+
+// ------------------------------------------------------------------ FP64 in fixed point
+// FP64 adds and multiplies run at under two lanes a clock per SM on this part, and a shared
+// FP64 atomic at 20 clocks a warp; 32-bit integer multiply-adds run at 64 lanes a clock. So
+// FP64 grids of orders 2 to 5 are deposited in integers: offsets in the cell as 63-bit
+// fractions, weights as 62-bit ones (two words of 31 bits), values scaled by the largest
+// exponent of their field to 62 bits, and each contribution, a 62-bit integer, split into
+// words of 22, 22 and 18 bits that are summed by 32-bit shared adds. A contribution is off
+// by a few units of 2^-61 of the largest value, where an FP64 product and an FP64 sum round
+// at 2^-53 of their own; the sums are exact and do not depend on the order. The low words
+// take up to 1023 adds, then their carries are moved up. Nodes become FP64 by one rounding.
+constexpr int kIxLow = 22;         // bits of the two low words
+constexpr uint32_t kIxChunk = 1016;  // particles between carries (a multiple of 8, below 2^10)
+
+// (a b) / 2^63 of 63-bit fractions (at most 2^63 itself)
+__device__ __forceinline__ unsigned long long mul63(unsigned long long a, unsigned long long b)
+{
+    return __umul64hi(a, b) << 1;
+}
+
+// Order-M B-spline weights as 63-bit fractions for the offset t (a fraction, at most 2^63);
+// the nodes as in bspline_weights.
+template <int M>
+__device__ __forceinline__ void fixed_weights(unsigned long long t, unsigned long long (&w)[M], int &first)
+{
+    using u64 = unsigned long long;
+    constexpr u64 one = 1ull << 63, half = 1ull << 62;
+    constexpr u64 sixth = 0x2aaaaaaaaaaaaaabull;  // 2^64 / 6
+    constexpr u64 c24 = 0x0aaaaaaaaaaaaaabull;    // 2^64 / 24
+    const bool up = t >= half;
+    if constexpr (M == 2) {
+        first = 0;
+        w[0] = one - t;
+        w[1] = t;
+    } else if constexpr (M == 4) {
+        first = -1;
+        const u64 v = one - t, t2 = mul63(t, t), t3 = mul63(t2, t), v2 = mul63(v, v), v3 = mul63(v2, v);
+        constexpr u64 two_thirds = 0x5555555555555555ull;
+        w[0] = __umul64hi(v3, sixth);
+        w[1] = two_thirds - t2 + (t3 >> 1);
+        w[2] = two_thirds - v2 + (v3 >> 1);
+        w[3] = __umul64hi(t3, sixth);
+    } else {
+        // b = 1/2 + d and a = 1/2 - d, d the offset from the nearest node
+        const u64 b = up ? t - half : t + half, a = one - b, d = up ? one - t : t;
+        const u64 a2 = mul63(a, a), b2 = mul63(b, b), d2 = mul63(d, d);
+        if constexpr (M == 3) {
+            first = up ? 0 : -1;
+            w[0] = a2 >> 1;
+            w[1] = half + (half >> 1) - d2;
+            w[2] = b2 >> 1;
+        } else {
+            first = up ? -1 : -2;
+            const u64 a4 = mul63(a2, a2), b4 = mul63(b2, b2);
+            auto mid = [](u64 x, u64 x2, u64 x4) {  // (1 + 4x + 6x^2 + 4x^3 - 4x^4) / 24
+                const u64 x3 = mul63(x2, x);
+                return (c24 >> 1) + (x2 >> 2) + __umul64hi(x + x3 - x4, sixth);
+            };
+            w[0] = __umul64hi(a4, c24);
+            w[1] = mid(a, a2, a4);
+            w[2] = 0x4caaaaaaaaaaaaabull - (d2 >> 1) - (d2 >> 3) + (mul63(d2, d2) >> 2);  // 115/192 - 5/8 d^2 + d^4/4
+            w[3] = mid(b, b2, b4);
+            w[4] = __umul64hi(b4, c24);
+        }
+    }
+}
+
+// x 2^(62 - shift) / 2^(biased - 1022) rounded, for a finite x whose biased exponent is at
+// most `biased`: below 2^(62 - shift) in magnitude
+__device__ __forceinline__ long long fixed_value(double x, int biased, int shift)
+{
+    const long long bits = __double_as_longlong(x);
+    const int e = static_cast<int>(bits >> 52) & 0x7ff;
+    long long m = (bits & ((1ll << 52) - 1)) | (e ? 1ll << 52 : 0ll);
+    const int left = (e ? e : 1) - max(biased, 1) + 9 - shift;
+    if (left >= 0) m <<= left;
+    else m = left < -62 ? 0 : (m + (1ll << (-left - 1))) >> -left;
+    return bits < 0 ? -m : m;
+}
+
+// The node sum hi 2^44 + low (0 <= low < 2^44) times 2^scale as FP64, rounded once
+__device__ __forceinline__ double fixed_to_double(int hi, long long low, int scale)
+{
+    // above 62 bits the lowest bits are dropped, which leaves 61
+    const int drop = max(0, 32 - __clz(hi < 0 ? ~hi : hi) - 18);
+    const long long v = (static_cast<long long>(hi) << (44 - drop)) + (low >> drop);
+    scale += drop;
+    if (v == 0) return 0.0;
+    const bool neg = v < 0;
+    unsigned long long m = neg ? 0ull - static_cast<unsigned long long>(v) : static_cast<unsigned long long>(v);
+    const int lz = __clzll(static_cast<long long>(m));
+    const int e = 1023 + 63 - lz + scale;  // biased exponent
+    m <<= lz;                              // the leading one at bit 63
+    if (e < 1 || e > 2045) return scalbn(static_cast<double>(v), scale);
+    const unsigned long long rest = m & 0x7ff, q = m >> 11;
+    unsigned long long r = (q & ((1ull << 52) - 1)) | (static_cast<unsigned long long>(e) << 52);
+    r += (rest > 0x400 || (rest == 0x400 && (q & 1))) ? 1 : 0;  // a carry moves the exponent up
+    return __longlong_as_double(static_cast<long long>(r | (neg ? 1ull << 63 : 0ull)));
+}
+
+// Three shared-memory adds at byte offsets OFF + j * FS from addr (immediates).
+template <int OFF, int FS>
+__device__ __forceinline__ void red3(unsigned addr, int v0, int v1, int v2)
+{
+    asm volatile(
+        "red.shared.add.s32 [%0+%4], %1;\n\t"
+        "red.shared.add.s32 [%0+%5], %2;\n\t"
+        "red.shared.add.s32 [%0+%6], %3;" ::"r"(addr), "r"(v0), "r"(v1), "r"(v2), "n"(OFF), "n"(OFF + FS), "n"(OFF + 2 * FS));
+}
+
+// Layout and lane mapping of the fixed-point deposit: 4 fields of 3 words, TNP ints each; one
+// particle per warp as in CoopLanes. Order 4: lane (dx, dy, h), four z nodes, fields 2h and
+// 2h + 1; order 5: lane (dx, dy) of 25, all z and fields; order 3: lane (dx, dy, dz) of 27,
+// all fields; order 2: lane (dx, dy, dz, field). The pitches put the lanes' nodes in
+// different banks (checked below); the lanes without a node take the free banks and a weight
+// of zero.
+template <int M, int T0, int T1, int T2>
+struct IxLanes {
+    static constexpr int RW = M == 2 ? T2 : M == 3 ? (T2 == 8 ? 11 : 18) : M == 4 && T2 == 8 ? 8 : T2 + 1;
+    static constexpr int PX =
+        T1 * RW + (M == 2 ? (T2 == 8 ? 16 : 2) : M == 3 ? (T2 == 8 ? 1 : 5) : M == 4 ? (T2 == 8 ? 1 : 0) : T2 == 8 ? 2 : 3);
+    static constexpr int TNP = T0 * PX + (M == 2 ? (T2 == 8 ? 2 : 4) : M == 4 ? 2 : 0);
+    static constexpr int FRONT = (5 * (PX + RW + 1) + 3) / 4 * 4;
+    static constexpr int BACK = 5 * (PX + RW + 1) + 32;
+    static constexpr size_t bytes = size_t(FRONT + 12 * TNP + BACK) * sizeof(int);
+    static constexpr int NZ = M >= 4 ? M : 1;
+    static constexpr int NF = M == 2 ? 1 : M == 4 ? 2 : 4;
+    static constexpr int USED = M == 3 ? 27 : M == 5 ? 25 : 32;
+    static constexpr int WQ = 6 * M;                 // staged words per particle: 3 M weights of two words,
+    static constexpr int QQ = (WQ + 3) / 4 * 4;      // four values of two words, the first node
+    static constexpr int STRIDE = QQ + 12;
+    static constexpr int NB = 8;
+    __host__ __device__ static constexpr int dx(int l) { return M == 2 ? l & 1 : M == 3 ? l / 9 : M == 4 ? (l >> 2) & 3 : l / 5; }
+    __host__ __device__ static constexpr int dy(int l) { return M == 2 ? (l >> 1) & 1 : M == 3 ? (l / 3) % 3 : M == 4 ? l & 3 : l % 5; }
+    __host__ __device__ static constexpr int dz(int l) { return M == 2 ? (l >> 2) & 1 : M == 3 ? l % 3 : 0; }
+    __host__ __device__ static constexpr int field(int l) { return M == 2 ? l >> 3 : M == 4 ? 2 * (l >> 4) : 0; }
+    __host__ __device__ static constexpr int node_offset(int l)
+    {
+        return dx(l) * PX + dy(l) * RW + dz(l) + 3 * field(l) * TNP;
+    }
+    static constexpr unsigned free_banks()
+    {
+        unsigned seen = 0;
+        for (int l = 0; l < USED; ++l) seen |= 1u << (node_offset(l) & 31);
+        return ~seen;
+    }
+    static constexpr bool banks_distinct()
+    {
+        int n = 0;
+        for (unsigned m = free_banks(); m; m &= m - 1) ++n;
+        return n == 32 - USED;
+    }
+    __device__ static int offset(int lane)
+    {
+        if (lane < USED) return node_offset(lane);
+        unsigned m = free_banks();
+        for (int l = USED; l < lane; ++l) m &= m - 1;
+        return __ffs(static_cast<int>(m)) - 1;
+    }
+    // the adds' nodes lie in the padded allocation (see fx_pads_cover)
+    static constexpr bool pads_cover()
+    {
+        constexpr int HL = (M % 2 == 0) ? M / 2 : (M + 1) / 2, HR = (M % 2 == 0) ? M / 2 - 1 : (M - 1) / 2;
+        constexpr int lo = -HL + bspline_first<M, float>(0.0f), up = HR - 1 + bspline_first<M, float>(0.5f) + M - 1;
+        return lo * (PX + RW + 1) >= -FRONT && (T0 + up) * PX + (T1 + up) * RW + T2 + up + 32 + 11 * TNP < 12 * TNP + BACK;
+    }
+    static_assert(banks_distinct() && pads_cover() && 3 * M * 2 <= WQ, "lanes in different banks, nodes in the pads");
+};
+
+// FP64 tile-gather deposit in fixed point (see above): one particle per warp, its weights
+// evaluated by four lanes (three axes and the values) for eight particles at a time, staged in
+// shared memory and read back by all lanes. Bound by integer issue. With FP64 products and
+// shared FP64 atomics 10^6 uniform particles on 128^3 took 3.57 ms, 10^6 in halos 19.1 ms;
+// in fixed point 0.94 and 1.37 ms.
+template <int M, int T0, int T1, int T2, int NT>
+__global__ void __launch_bounds__(NT)
+k_deposit_ix(const Record<double> *__restrict__ rec, const uint32_t *__restrict__ offsets,
+             const unsigned *__restrict__ qmax_bits, int ng, int sshift, double *__restrict__ grids, int64_t grid_elems,
+             int /*list_cap*/, bool /*sparse*/)
+{
+    using C = DepositCfg<double, M, T0, T1, T2, NT>;
+    using L = IxLanes<M, T0, T1, T2>;
+    constexpr int NW = NT / 32, TNP = L::TNP;
+    constexpr unsigned full = 0xffffffffu;
+    static_assert(L::bytes >= C::smem, "the FP64 accumulator fits too");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint32_t s_beg[C::MAXR];
+    __shared__ uint32_t s_pre[C::MAXR + 1];
+    __shared__ unsigned s_rowmax;
+    __shared__ __align__(16) int s_stage[NW][L::NB * L::STRIDE];
+    int top[4];  // biased exponent of the largest value of each field
+    bool finite = true;
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        top[f] = static_cast<int>(qmax_bits[f] >> 20);
+        finite = finite && top[f] < 0x7ff;
+    }
+    if (!finite || sshift != 0 || ng < C::R0 || ng < C::R1 || ng < T2 + C::HL + C::HR) {
+        // infinities and NaN, or a reach that wraps onto itself
+        deposit_fp64_tile<double, M, T0, T1, T2, NT, 0>(rec, offsets, ng, sshift, grids, grid_elems,
+                                                        reinterpret_cast<double *>(smem_raw), s_beg, s_pre);
+        return;
+    }
+    const int ntz = ng / T2, nty = ng / T1;
+    int tile = blockIdx.x;
+    const int tz = tile % ntz;
+    tile /= ntz;
+    const int ty = tile % nty, tx = tile / nty;
+    const int t0 = tx * T0, t1 = ty * T1, t2 = tz * T2;
+    int *acc = reinterpret_cast<int *>(smem_raw) + L::FRONT;  // [4 fields][low, middle, high][TNP]
+    for (int k = threadIdx.x; k < 3 * TNP; k += NT) reinterpret_cast<int4 *>(acc)[k] = make_int4(0, 0, 0, 0);
+    if (threadIdx.x == 0) s_rowmax = 0;
+    const uint32_t total = build_ranges<C>(offsets, ng, sshift, t0, t1, t2, T2, s_beg, s_pre);
+    for (int r = threadIdx.x; 2 * r + 1 < C::MAXR + 1; r += NT) {
+        const uint32_t c = s_pre[2 * r + 2 <= C::MAXR ? 2 * r + 2 : C::MAXR] - s_pre[2 * r];
+        if (c) atomicMax(&s_rowmax, c);
+    }
+    __syncthreads();
+    // a node takes at most M x M rows' particles: keep the high words below 2^31
+    const float bound = kMaxWeight3<M> * 1.0001f *
+                        fminf(static_cast<float>(M * M) * static_cast<float>(s_rowmax), static_cast<float>(total));
+    int shift = 0;
+    while (bound > static_cast<float>(8000u << shift) && shift < 18) ++shift;
+
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, a = lane & 3, sub = lane >> 2;
+    const int corner = a == 0 ? t0 : a == 1 ? t1 : t2, edge = a == 0 ? T0 : a == 1 ? T1 : T2;
+    const int pitch = a == 0 ? L::PX : a == 1 ? L::RW : a == 2 ? 1 : 0;
+    const bool node = lane < L::USED;
+    const int offset = L::offset(lane);
+    int *const stage = s_stage[warp];
+    const unsigned mine = static_cast<unsigned>(__cvta_generic_to_shared(acc)) + 4 * offset;
+    const int *const sx = stage + 2 * (node ? L::dx(lane) : 0), *const sy = stage + 2 * M + 2 * (node ? L::dy(lane) : 0),
+              *const sz = stage + 4 * M + 2 * (node ? L::dz(lane) : 0), *const sq = stage + L::QQ + 2 * L::field(lane);
+
+    for (uint32_t c0 = 0; c0 < total; c0 += kIxChunk) {
+        const uint32_t cnt = min(total - c0, kIxChunk);
+        if (c0) {  // carries: after at most 1023 adds
+            __syncthreads();
+            for (int k = threadIdx.x; k < 4 * TNP; k += NT) {
+                int *w = acc + (k / TNP) * 3 * TNP + k % TNP;
+                const unsigned lo = static_cast<unsigned>(w[0]);
+                const unsigned mid = static_cast<unsigned>(w[TNP]) + (lo >> kIxLow);
+                w[0] = static_cast<int>(lo & ((1u << kIxLow) - 1));
+                w[TNP] = static_cast<int>(mid & ((1u << kIxLow) - 1));
+                w[2 * TNP] += static_cast<int>(mid >> kIxLow);
+            }
+            __syncthreads();
+        }
+        const uint32_t share = ((cnt + NW - 1) / NW + L::NB - 1) / L::NB * L::NB;
+        const uint32_t lo = min(cnt, warp * share), hi = min(cnt, lo + share);
+        int slot = lo + sub < hi ? find_slot<C::MAXR>(s_pre, c0 + lo + sub) : 0;
+        double v = 0.0, q[4] = {0.0, 0.0, 0.0, 0.0};
+        auto fetch = [&](uint32_t at) {
+            if (at + sub < hi) {
+                const uint32_t p = c0 + at + sub;
+                while (p >= s_pre[slot + 1]) ++slot;
+                const Record<double> *r = rec + s_beg[slot] + (p - s_pre[slot]);
+                v = reinterpret_cast<const double *>(r)[a];
+                if (a == 3) q[0] = r->q.x, q[1] = r->q.y, q[2] = r->q.z, q[3] = r->q.w;
+            }
+        };
+        fetch(lo);
+        for (uint32_t at = lo; at < hi; at += L::NB) {
+            const int nb = static_cast<int>(min(hi - at, static_cast<uint32_t>(L::NB)));
+            const int packed = __shfl_sync(full, unpack_cell(v), lane | 3);
+            // the offset in the cell (in [0, 1]) as a 63-bit fraction
+            const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(a == 3 ? 0.0 : v));
+            const int e = static_cast<int>(bits >> 52) - 1012;
+            unsigned long long t = (bits & ((1ull << 52) - 1)) | 1ull << 52;
+            t = e >= 0 ? t << e : e > -53 ? t >> -e : 0ull;
+            unsigned long long w[M];
+            int first;
+            fixed_weights<M>(t, w, first);
+            int d = ((packed >> (10 * min(a, 2))) & 1023) - corner;
+            d = d < -C::HL ? d + ng : (d >= edge + C::HR ? d - ng : d);
+            d += first;
+            int word = d * pitch;
+            word += __shfl_xor_sync(full, word, 1);
+            word += __shfl_xor_sync(full, word, 2);
+            int *const st = stage + sub * L::STRIDE;
+            if (sub < nb) {
+                if (a < 3) {
+#pragma unroll
+                    for (int k = 0; k < M; ++k) {
+                        // 62 bits (one itself just below), zero outside the tile
+                        const bool in = static_cast<unsigned>(d + k) < static_cast<unsigned>(edge);
+                        const unsigned long long x = in ? min(w[k] >> 1, (1ull << 62) - 1) : 0ull;
+                        *reinterpret_cast<int2 *>(st + 2 * (a * M + k)) =
+                            make_int2(static_cast<int>(x >> 31), static_cast<int>(x & 0x7fffffffu));
+                    }
+                } else {
+#pragma unroll
+                    for (int f = 0; f < 4; ++f) {
+                        const long long x = fixed_value(q[f], top[f], shift);
+                        *reinterpret_cast<int2 *>(st + L::QQ + 2 * f) =
+                            make_int2(static_cast<int>(x >> 31), static_cast<int>(x & 0x7fffffffll));
+                    }
+                    st[L::QQ + 8] = word;
+                }
+            }
+            __syncwarp();
+            fetch(at + L::NB);
+#pragma unroll 2
+            for (int p = 0; p < nb; ++p) {
+                const int o = p * L::STRIDE;
+                const int2 x = *reinterpret_cast<const int2 *>(sx + o), y = *reinterpret_cast<const int2 *>(sy + o);
+                const unsigned addr = mine + static_cast<unsigned>(4 * stage[L::QQ + 8 + o]);
+                auto mul = [](int2 u, int2 w) {  // u w / 2^62 of values in words of 31 bits
+                    const long long cross = static_cast<long long>(u.x) * w.y + static_cast<long long>(u.y) * w.x;
+                    return static_cast<long long>(u.x) * w.x + (cross >> 31);
+                };
+                auto split = [](long long u) {
+                    return make_int2(static_cast<int>(u >> 31), static_cast<int>(u & 0x7fffffffll));
+                };
+                int2 xy = split(mul(x, y));
+                if (L::USED < 32 && !node) xy = make_int2(0, 0);
+                static_for<L::NZ>([&](auto kc) {
+                    constexpr int k = decltype(kc)::value;
+                    const int2 ww = split(mul(xy, *reinterpret_cast<const int2 *>(sz + o + 2 * k)));
+                    static_for<L::NF>([&](auto fc) {
+                        constexpr int f = decltype(fc)::value;
+                        const long long c = mul(*reinterpret_cast<const int2 *>(sq + o + 2 * f), ww);
+                        if (!PK_IN(stage[L::QQ + 8 + o] + offset + L::FRONT + k + 3 * f * TNP + 2 * TNP,
+                                   L::FRONT + 12 * TNP + L::BACK, kChkShared))
+                            return;
+                        red3<4 * (k + 3 * f * TNP), 4 * TNP>(addr, static_cast<int>(c) & ((1 << kIxLow) - 1),
+                                                             static_cast<int>(c >> kIxLow) & ((1 << kIxLow) - 1),
+                                                             static_cast<int>(c >> (2 * kIxLow)));
+                    });
+                });
+            }
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < C::TN; k += NT) {
+        const int l2 = k % T2, l01 = k / T2;
+        const int l1 = l01 % T1, l0 = l01 / T1;
+        const int64_t gi = (static_cast<int64_t>(t0 + l0) * ng + (t1 + l1)) * (ng + 2) + t2 + l2;
+        if (!PK_IN(gi, grid_elems, kChkGrid)) continue;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            const int *w = acc + 3 * f * TNP + l0 * L::PX + l1 * L::RW + l2;
+            const long long low = (static_cast<long long>(static_cast<unsigned>(w[TNP])) << kIxLow) +
+                                  static_cast<unsigned>(w[0]);
+            grids[f * grid_elems + gi] =
+                fixed_to_double(w[2 * TNP] + static_cast<int>(low >> 44), low & ((1ll << 44) - 1),
+                                max(top[f], 1) - 1022 - 62 + shift);
+        }
     }
 }
 
@@ -2307,6 +2672,9 @@ cudaError_t launch_deposit_t(const AssignPlan &pl, const uint32_t *offsets, cons
         kern = k_deposit_fx<M, T0, T1, T2, NT, BLR>;
         list_cap = pl.list_cap;
         smem = FxLayout<M, T0, T1, T2>::bytes(list_cap);
+    } else if constexpr (M >= 2 && M <= 5 && BLR == 0 && T0 == 8) {
+        kern = k_deposit_ix<M, T0, T1, T2, NT>;
+        smem = IxLanes<M, T0, T1, T2>::bytes;
     } else {
         kern = k_deposit<T, M, T0, T1, T2, NT, BLR>;
     }
