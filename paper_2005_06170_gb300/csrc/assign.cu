@@ -314,6 +314,18 @@ struct LaneMoments {
             sum[k] += x;
         }
     }
+    // adds another lane's sums (FP32: the pairs exactly, to 2^-48) and maxima
+    __device__ __forceinline__ void merge(const LaneMoments &o)
+    {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            T hi = sum[k], lo = -cmp[k];
+            pair_add(hi, lo, o.sum[k], -o.cmp[k]);
+            sum[k] = hi, cmp[k] = -lo;
+        }
+#pragma unroll
+        for (int f = 0; f < 4; ++f) qmax[f] = max(qmax[f], o.qmax[f]);
+    }
     __device__ __forceinline__ void add(T m, T v0, T v1, T v2)
     {
         if constexpr (MASS) {
@@ -459,35 +471,43 @@ k_moments(const T *__restrict__ vx, const T *__restrict__ vy, const T *__restric
 
 // FP32 interleaved (n, 3) velocities, 16-byte aligned: four particles per thread read
 // as three 128-bit loads ((v0x v0y v0z v1x) (v1y v1z v2x v2y) (v2z v3x v3y v3z)), and
-// four masses as one. The n % 4 last particles are added by the first lanes of block 0.
+// four masses as one. The particles are dealt to `lanes` sums, lane v taking the quads v,
+// v + lanes, ..., and lane v < 32 the v-th of the n % 4 last particles, whatever the number
+// of threads (a thread takes several lanes and merges their pairs): a compensated sum of
+// values that cancel, such as the momentum of a catalogue without bulk flow, depends on how
+// they are dealt, and the size of the launch should not matter.
 template <bool MASS>
 __global__ void __launch_bounds__(kMomentThreads)
-k_moments_v3(const float *__restrict__ v, const float *__restrict__ mass, int64_t n, double *__restrict__ partials,
-             unsigned *__restrict__ qmax_bits, unsigned *__restrict__ done, double *__restrict__ out)
+k_moments_v3(const float *__restrict__ v, const float *__restrict__ mass, int64_t n, int64_t lanes,
+             double *__restrict__ partials, unsigned *__restrict__ qmax_bits, unsigned *__restrict__ done,
+             double *__restrict__ out)
 {
-    LaneMoments<float, MASS> lm;
     const int64_t nq = n / 4;
     const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x;
     const float4 *v4 = reinterpret_cast<const float4 *>(v);
     const float4 *m4 = reinterpret_cast<const float4 *>(mass);
-    for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < nq; q += step) {
-        const float4 a = v4[3 * q], b = v4[3 * q + 1], c = v4[3 * q + 2];
-        float4 mm = make_float4(1.f, 1.f, 1.f, 1.f);
-        if constexpr (MASS) mm = m4[q];
-        lm.add(mm.x, a.x, a.y, a.z);
-        lm.add(mm.y, a.w, b.x, b.y);
-        lm.add(mm.z, b.z, b.w, c.x);
-        lm.add(mm.w, c.y, c.z, c.w);
-    }
-    if (blockIdx.x == 0 && threadIdx.x < 32) {
-        const int64_t i = 4 * nq + threadIdx.x;
-        if (i < n) {
+    const int64_t used = nq > 32 ? (nq < lanes ? nq : lanes) : 32;  // the other lanes are empty
+    LaneMoments<float, MASS> all;
+    for (int64_t vl = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; vl < used; vl += step) {
+        LaneMoments<float, MASS> lm;
+        for (int64_t q = vl; q < nq; q += lanes) {
+            const float4 a = v4[3 * q], b = v4[3 * q + 1], c = v4[3 * q + 2];
+            float4 mm = make_float4(1.f, 1.f, 1.f, 1.f);
+            if constexpr (MASS) mm = m4[q];
+            lm.add(mm.x, a.x, a.y, a.z);
+            lm.add(mm.y, a.w, b.x, b.y);
+            lm.add(mm.z, b.z, b.w, c.x);
+            lm.add(mm.w, c.y, c.z, c.w);
+        }
+        const int64_t i = 4 * nq + vl;
+        if (vl < 32 && i < n) {
             float m = 1.f;
             if constexpr (MASS) m = mass[i];
             lm.add(m, v[3 * i], v[3 * i + 1], v[3 * i + 2]);
         }
+        all.merge(lm);
     }
-    finish_moments<float, MASS>(lm, n, partials, qmax_bits, done, out);
+    finish_moments<float, MASS>(all, n, partials, qmax_bits, done, out);
 }
 
 // ------------------------------------------------------------------ scatter
@@ -2867,8 +2887,13 @@ void scatter_and_moments(const pkmom_catalog &cat, const AssignPlan &pl, T scale
         const bool v3 = cat.stride == 3 && vy == vx + 1 && vz == vx + 2 && reinterpret_cast<uintptr_t>(vx) % 16 == 0 &&
                         reinterpret_cast<uintptr_t>(mass) % 16 == 0;
         if (v3) {
-            if (mass) k_moments_v3<true><<<blocks, kMomentThreads, 0, s>>>(vx, mass, cat.n, partials, qmax, done, moments_dev);
-            else k_moments_v3<false><<<blocks, kMomentThreads, 0, s>>>(vx, mass, cat.n, partials, qmax, done, moments_dev);
+            const int64_t lanes = static_cast<int64_t>(pl.hist_blocks) * kMomentThreads;
+            if (mass)
+                k_moments_v3<true><<<blocks, kMomentThreads, 0, s>>>(vx, mass, cat.n, lanes, partials, qmax, done,
+                                                                     moments_dev);
+            else
+                k_moments_v3<false><<<blocks, kMomentThreads, 0, s>>>(vx, mass, cat.n, lanes, partials, qmax, done,
+                                                                      moments_dev);
             return;
         }
     }
