@@ -2235,15 +2235,15 @@ __device__ __forceinline__ void home_pair(unsigned acc_s, const Record<float> (&
     for (int j = 0; j < CP; ++j) qp[j][0] = f2_pack(q[j][0], q[j][1]), qp[j][1] = f2_pack(q[j][2], q[j][3]);
     const f32x2 mg = f2_pack(kMagic, kMagic);
     // buffer index of node (cx - 1 + dx, cy - 1 + dy, CP m - 1 + i) is (cx + dx) PX + (cy + dy) PY + CP m + i.
-    // The 4 x 4 node columns are two rolled loops (a short body for the instruction
-    // cache); the weights of the current dx and dy are kept in slot 0 by rotating them.
+    // The dx loop is rolled (a short body for the instruction cache): the weights of the
+    // current dx are kept in slot 0 by rotating them.
     // the lane's last node (3, 3 node columns on) must lie in the buffer
     if (!PK_IN((cx + 3) * kHomePX + (cy + 3) * kHomePY + CP * m + CP + 2, kHomeField, kChkShared)) return;
     unsigned base = acc_s + 4u * static_cast<unsigned>(cx * kHomePX + cy * kHomePY + CP * m);
 #pragma unroll 1
     for (int dx = 0; dx < 4; ++dx) {
-#pragma unroll 1
-        for (int dy = 0; dy < 4; ++dy) {
+        static_for<4>([&](auto dyc) {
+            constexpr int dy = decltype(dyc)::value;
             unsigned a[CP + 3][4];
             static_for<CP + 3>([&](auto ic) {
                 constexpr int i = decltype(ic)::value;
@@ -2253,7 +2253,7 @@ __device__ __forceinline__ void home_pair(unsigned acc_s, const Record<float> (&
             });
 #pragma unroll
             for (int j = 0; j < CP; ++j) {
-                const float w01 = wx[j][0] * wy[j][0];
+                const float w01 = wx[j][0] * wy[j][dy];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const float ww = w01 * wz[j][k];
@@ -2265,18 +2265,12 @@ __device__ __forceinline__ void home_pair(unsigned acc_s, const Record<float> (&
                     a[j + k][3] += static_cast<unsigned>(t23 >> 32);
                 }
             }
-            const unsigned b = base + 4u * static_cast<unsigned>(dy * kHomePY);
             static_for<CP + 3>([&](auto ic) {
                 constexpr int i = decltype(ic)::value;
-                red4<4 * i, 4 * kHomeField>(b, static_cast<int>(a[i][0]), static_cast<int>(a[i][1]),
-                                            static_cast<int>(a[i][2]), static_cast<int>(a[i][3]));
+                red4<4 * (dy * kHomePY + i), 4 * kHomeField>(base, static_cast<int>(a[i][0]), static_cast<int>(a[i][1]),
+                                                             static_cast<int>(a[i][2]), static_cast<int>(a[i][3]));
             });
-#pragma unroll
-            for (int j = 0; j < CP; ++j) {  // next dy in slot 0
-                const float t = wy[j][0];
-                wy[j][0] = wy[j][1], wy[j][1] = wy[j][2], wy[j][2] = wy[j][3], wy[j][3] = t;
-            }
-        }
+        });
 #pragma unroll
         for (int j = 0; j < CP; ++j) {  // next dx in slot 0
             const float t = wx[j][0];
@@ -2434,30 +2428,35 @@ k_deposit_home(const Record<float> *__restrict__ rec, const uint32_t *__restrict
     const float sc0 = s_scale[0], sc1 = s_scale[1], sc2 = s_scale[2], sc3 = s_scale[3];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
-    // owned nodes to the grid, halo nodes to this tile's scratch; value(f, buffer index).
+    // owned nodes to the grid, halo nodes to this tile's scratch; value(f, buffer index); the
+    // node's place is found once for all fields.
     // Owned rows: eight lanes per (x, y) row, two z nodes each (8-byte stores: the rows
     // start at even offsets, ng + 2 and the tile corner being even, and the grids are
     // 16-byte aligned).
     float *h = halo + static_cast<int64_t>(blockIdx.x) * 4 * kHomeHalo;
-    auto emit = [&](int f, auto value) {
-        float *gf = grids + f * grid_elems;
+    auto emit = [&](auto fields, auto value) {  // fields: the first and one past the last
+        constexpr int F0 = decltype(fields)::value / 8, F1 = decltype(fields)::value % 8;
 #pragma unroll 2
         for (int rowi = threadIdx.x >> 3; rowi < kHomeT * kHomeT; rowi += kHomeNT / 8) {
             const int zp = 2 * (threadIdx.x & 7);
             const int x = rowi >> 4, y = rowi & 15;
             const int ab = (x + 1) * kHomePX + (y + 1) * kHomePY + zp + 1;
             const int64_t gi = (static_cast<int64_t>(t0 + x) * ng + (t1 + y)) * (ng + 2) + t2 + zp;
-            if (PK_IN(gi + 1, grid_elems, kChkGrid) && PK_IN(ab + 1, kHomeField, kChkShared))
-                *reinterpret_cast<float2 *>(gf + gi) = make_float2(value(ab), value(ab + 1));
+            if (!PK_IN(gi + 1, grid_elems, kChkGrid) || !PK_IN(ab + 1, kHomeField, kChkShared)) continue;
+#pragma unroll
+            for (int f = F0; f < F1; ++f)
+                *reinterpret_cast<float2 *>(grids + f * grid_elems + gi) = make_float2(value(f, ab), value(f, ab + 1));
         }
         for (int k = threadIdx.x; k < kHomeHalo; k += kHomeNT) {
             int bx, by, bz;
             home_halo_node(k, bx, by, bz);
             const int ai = bx * kHomePX + by * kHomePY + bz;
-            if (PK_IN(static_cast<int64_t>(blockIdx.x) * 4 * kHomeHalo + f * kHomeHalo + k,
-                      static_cast<int64_t>(gridDim.x) * 4 * kHomeHalo, kChkHalo) &&
-                PK_IN(ai, kHomeField, kChkShared))
-                h[f * kHomeHalo + k] = value(ai);
+            if (!PK_IN(static_cast<int64_t>(blockIdx.x) * 4 * kHomeHalo + (F1 - 1) * kHomeHalo + k,
+                       static_cast<int64_t>(gridDim.x) * 4 * kHomeHalo, kChkHalo) ||
+                !PK_IN(ai, kHomeField, kChkShared))
+                continue;
+#pragma unroll
+            for (int f = F0; f < F1; ++f) h[f * kHomeHalo + k] = value(f, ai);
         }
     };
 
@@ -2478,19 +2477,15 @@ k_deposit_home(const Record<float> *__restrict__ rec, const uint32_t *__restrict
             if (pass == 0) home_cells_path<0>(rec, offsets, ng, t0, t1, t2, smem_raw, limbs, s_fine);
             else home_cells_path<2>(rec, offsets, ng, t0, t1, t2, smem_raw, limbs, s_fine);
             __syncthreads();
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const int f = 2 * pass + k;
-                const float inv = 1.0f / s_fine[f];  // exact: a power of two
-                const auto *a64 = reinterpret_cast<const long long *>(smem_raw) + k * kHomeField;
-                const int *a32 = acc + 2 * k * kHomeField;
-                emit(f, [&](int ai) {
-                    const long long v = limbs ? static_cast<long long>(a32[kHomeField + ai]) * 65536 +
-                                                    static_cast<unsigned>(a32[ai])
-                                              : a64[ai];
-                    return static_cast<float>(v) * inv;
-                });
-            }
+            auto value = [&](int f, int ai) {
+                const int k = f & 1;
+                const long long v = limbs ? static_cast<long long>(acc[(2 * k + 1) * kHomeField + ai]) * 65536 +
+                                                static_cast<unsigned>(acc[2 * k * kHomeField + ai])
+                                          : reinterpret_cast<const long long *>(smem_raw)[k * kHomeField + ai];
+                return static_cast<float>(v) * (1.0f / s_fine[f]);  // exact: a power of two
+            };
+            if (pass == 0) emit(std::integral_constant<int, 0 * 8 + 2>{}, value);
+            else emit(std::integral_constant<int, 2 * 8 + 4>{}, value);
         }
         return;
     }
@@ -2546,38 +2541,30 @@ k_deposit_home(const Record<float> *__restrict__ rec, const uint32_t *__restrict
             }
             home_pair(acc_s, r, has, cx, cy, m, sc0, sc1, sc2, sc3);
             // second and later particles of the cells: the per-warp queue, 32 at a time
-#pragma unroll 1
-            for (int k = 0; k < CP; ++k) {
-                uint32_t next = o[k] + 1, extra = has[k] ? o[k + 1] - o[k] - 1 : 0u;
-                while (__any_sync(0xffffffffu, extra > 0u)) {
-                    const bool more = extra > 0u;
-                    const unsigned mk = __ballot_sync(0xffffffffu, more);
-                    if (more) {
-                        q[qn + __popc(mk & ((1u << lane) - 1u))] = next;
-                        ++next;
-                        --extra;
-                    }
-                    qn += __popc(mk);
+            static_assert(CP == 2, "the lane's two cells");
+            const uint32_t n0 = has[0] ? o[1] - o[0] - 1u : 0u, n1 = has[1] ? o[2] - o[1] - 1u : 0u;
+            for (uint32_t i = 0;; ++i) {
+                const bool more = i < n0 + n1;
+                const unsigned mk = __ballot_sync(0xffffffffu, more);
+                if (!mk) break;
+                if (more) q[qn + __popc(mk & ((1u << lane) - 1u))] = i < n0 ? o[0] + 1u + i : o[1] + 1u + (i - n0);
+                qn += __popc(mk);
+                __syncwarp();
+                if (qn >= 32) {
+                    home_listed(acc, rec, q[lane], t0, t1, t2, sc0, sc1, sc2, sc3);
                     __syncwarp();
-                    if (qn >= 32) {
-                        home_listed(acc, rec, q[lane], t0, t1, t2, sc0, sc1, sc2, sc3);
-                        __syncwarp();
-                        if (lane < qn - 32) q[lane] = q[lane + 32];
-                        qn -= 32;
-                        __syncwarp();
-                    }
+                    if (lane < qn - 32) q[lane] = q[lane + 32];
+                    qn -= 32;
+                    __syncwarp();
                 }
             }
         }
         if (lane < qn) home_listed(acc, rec, q[lane], t0, t1, t2, sc0, sc1, sc2, sc3);
     }
     __syncthreads();
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-        const float inv = 1.0f / s_scale[f];  // exact: a power of two
-        const int *a = acc + f * kHomeField;
-        emit(f, [&](int ai) { return static_cast<float>(a[ai]) * inv; });
-    }
+    const float inv[4] = {1.0f / sc0, 1.0f / sc1, 1.0f / sc2, 1.0f / sc3};  // exact: powers of two
+    emit(std::integral_constant<int, 0 * 8 + 4>{},
+         [&](int f, int ai) { return static_cast<float>(acc[f * kHomeField + ai]) * inv[f]; });
 }
 
 // Owned nodes within reach of a neighbouring tile's particles (local index 0, 1 or 15
