@@ -1227,10 +1227,12 @@ struct CellPieces {
 // magnitude: one FFMA against 1.5 * 2^23) and added as an integer; the chunk sum is then
 // rounded to the tile scale by a right shift of sf - st bits. Integer sums: the result
 // does not depend on the order in which the sort left the cell's particles.
+// With z >= 0 only the particles of cells at that z count (keys of several cells), at most
+// kCellFlush of them; returns where the next chunk starts.
 template <int F0 = 0, int NF = 4>
-__device__ __forceinline__ void cell_chunk(const Record<float> *__restrict__ rec, uint32_t i0, uint32_t i1,
+__device__ __forceinline__ uint32_t cell_chunk(const Record<float> *__restrict__ rec, uint32_t i0, uint32_t i1,
                                            const CellPieces &pc, const float (&fine)[4], const int (&shift)[4],
-                                           int (&a)[NF], int (&b)[NF])
+                                           int (&a)[NF], int (&b)[NF], int z = -1)
 {
     constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
     constexpr int kMagicBits = 0x4B400000;
@@ -1249,6 +1251,13 @@ __device__ __forceinline__ void cell_chunk(const Record<float> *__restrict__ rec
         }
     };
     uint32_t i = i0;
+    if (z >= 0) {
+        for (int n = 0; i < i1 && n < kCellFlush; ++i) {
+            const Record<float> r = load_record(rec + i);
+            if ((unpack_cell(r.u.w) >> 20) == z) add(r), ++n;  // warp-uniform
+        }
+        i1 = i;
+    }
     for (; i + 4 <= i1; i += 4) {  // four loads in flight
         const Record<float> r0 = load_record(rec + i), r1 = load_record(rec + i + 1), r2 = load_record(rec + i + 2),
                             r3 = load_record(rec + i + 3);
@@ -1263,6 +1272,7 @@ __device__ __forceinline__ void cell_chunk(const Record<float> *__restrict__ rec
         a[f] = round_shift(sa[f], shift[F0 + f]);
         b[f] = round_shift(sb[f], shift[F0 + f]);
     }
+    return i1;
 }
 
 // Fixed-point scales of a tile: 2^st with (bound of any node sum) * 2^st < 2^30, and,
@@ -1286,8 +1296,8 @@ __device__ __forceinline__ void tile_scales(float bound, float cmax, bool cells,
 
 template <int T0, int T1, int T2, int NT>
 __device__ __forceinline__ void deposit_cells_path(const Record<float> *__restrict__ rec,
-                                                   const uint32_t *__restrict__ offsets, int ng, int t0, int t1, int t2,
-                                                   int *acc, int fstride, int px, int rw, const float *s_fine,
+                                                   const uint32_t *__restrict__ offsets, int ng, int sshift, int t0,
+                                                   int t1, int t2, int *acc, int fstride, int px, int rw, const float *s_fine,
                                                    const int *s_shift)
 {
     constexpr int HL = 2, R0 = T0 + 3, R1 = T1 + 3, RZ = T2 + 3, NW = NT / 32;
@@ -1304,17 +1314,19 @@ __device__ __forceinline__ void deposit_cells_path(const Record<float> *__restri
     for (int c = warp; c < R0 * R1 * RZ; c += NW) {
         const int r = c / RZ, zz = c % RZ;
         const int cx = r / R1 - HL, cy = r % R1 - HL, cz = zz - HL;  // cell relative to the tile
+        const int z = wrapi(t2 + cz);
         const int64_t key =
-            (static_cast<int64_t>(wrapi(t0 + cx)) * ng + wrapi(t1 + cy)) * ng + wrapi(t2 + cz);
+            (static_cast<int64_t>(wrapi(t0 + cx)) * ng + wrapi(t1 + cy)) * (ng >> sshift) + (z >> sshift);
         const uint32_t beg = offsets[key], end = offsets[key + 1];
         if (beg == end) continue;
         const int lxa = cx - 1 + dxl, lxb = lxa + 2, ly = cy - 1 + dy, lz = cz - 1 + dz;
         const bool yz = ly >= 0 && ly < T1 && lz >= 0 && lz < T2;
         const bool ina = yz && lxa >= 0 && lxa < T0, inb = yz && lxb >= 0 && lxb < T0;
         const int oa = lxa * px + ly * rw + lz, ob = (lxa + 2) * px + ly * rw + lz;
-        for (uint32_t i0 = beg; i0 < end; i0 += kCellFlush) {
+        for (uint32_t i0 = beg; i0 < end;) {
             int a[4], b[4];
-            cell_chunk(rec, i0, min(end, i0 + kCellFlush), pc, fine, shift, a, b);
+            i0 = sshift ? cell_chunk(rec, i0, end, pc, fine, shift, a, b, z)
+                        : cell_chunk(rec, i0, min(end, i0 + kCellFlush), pc, fine, shift, a, b);
 #pragma unroll
             for (int f = 0; f < 4; ++f) {
                 if (ina) atomicAdd(acc + f * fstride + oa, a[f]);
@@ -1470,19 +1482,33 @@ __device__ __forceinline__ void banked_particle(const Record<float> &r, int ng, 
         !PK_IN(b2 - LO, T2 + HI - LO + 1, kChkShared))
         return;
     const unsigned base = acc_s + 4u * static_cast<unsigned>(b0 * PX + b1 * RW + b2);
-    const float q0 = r.q.x * sc0, q1 = r.q.y * sc1, q2 = r.q.z * sc2, q3 = r.q.w * sc3;
+    const float qs[4] = {r.q.x * sc0, r.q.y * sc1, r.q.z * sc2, r.q.w * sc3};
+    f32x2 qp[4], zp[(M + 1) / 2];  // each value twice, the z weights in pairs (fma.rn.f32x2)
+#pragma unroll
+    for (int f = 0; f < 4; ++f) qp[f] = f2_pack(qs[f], qs[f]);
+#pragma unroll
+    for (int k = 0; k < M; k += 2) zp[k / 2] = f2_pack(w[2][k], k + 1 < M ? w[2][k + 1 < M ? k + 1 : k] : 0.0f);
+    const f32x2 mg = f2_pack(kMagic, kMagic);
     auto row = [&](auto k0c, auto k1c) {
         constexpr int k0 = decltype(k0c)::value, k1 = decltype(k1c)::value;
         const float w01 = w[0][k0] * w[1][k1];
-        auto node = [&](auto k2c) {
-            constexpr int k2 = decltype(k2c)::value;
-            const float ww = w01 * w[2][k2];
-            red4<4 * (k0 * PX + k1 * RW + k2), 4 * TNP>(base, __float_as_int(fmaf(q0, ww, kMagic)) - kMagicBits,
-                                                        __float_as_int(fmaf(q1, ww, kMagic)) - kMagicBits,
-                                                        __float_as_int(fmaf(q2, ww, kMagic)) - kMagicBits,
-                                                        __float_as_int(fmaf(q3, ww, kMagic)) - kMagicBits);
-        };
-        static_for<M>(node);
+        const f32x2 w2 = f2_pack(w01, w01);
+        static_for<(M + 1) / 2>([&](auto hc) {
+            constexpr int k2 = 2 * decltype(hc)::value;
+            const f32x2 ww = f2_mul(w2, zp[k2 / 2]);
+            f32x2 t[4];
+#pragma unroll
+            for (int f = 0; f < 4; ++f) t[f] = f2_fma(qp[f], ww, mg);
+            red4<4 * (k0 * PX + k1 * RW + k2), 4 * TNP>(base, static_cast<int>(t[0]) - kMagicBits,
+                                                        static_cast<int>(t[1]) - kMagicBits,
+                                                        static_cast<int>(t[2]) - kMagicBits,
+                                                        static_cast<int>(t[3]) - kMagicBits);
+            if constexpr (k2 + 1 < M)
+                red4<4 * (k0 * PX + k1 * RW + k2 + 1), 4 * TNP>(base, static_cast<int>(t[0] >> 32) - kMagicBits,
+                                                                static_cast<int>(t[1] >> 32) - kMagicBits,
+                                                                static_cast<int>(t[2] >> 32) - kMagicBits,
+                                                                static_cast<int>(t[3] >> 32) - kMagicBits);
+        });
     };
     static_for<M>([&](auto k0c) { static_for<M>([&](auto k1c) { row(k0c, k1c); }); });
 }
@@ -1594,7 +1620,12 @@ __device__ __forceinline__ void coop_deposit(const Record<float> *__restrict__ r
         d += first;
 #pragma unroll
         for (int k = 0; k < M; ++k) w[k] = static_cast<unsigned>(d + k) < static_cast<unsigned>(edge) ? w[k] : 0.0f;
-        int word = d * pitch;  // the first node, summed over the axes
+        // the first node, summed over the axes; node 0, with weights of zero, for a particle
+        // that does not reach the tile (keys of several cells)
+        const unsigned reaches = __ballot_sync(full, a == 3 || (d > -M && d < edge));
+        const bool in = ((reaches >> (lane & ~3)) & 15u) == 15u;
+        if (!in) w[0] = w[1] = w[2] = w[M - 1] = w[3] = 0.0f;
+        int word = in ? d * pitch : 0;
         word += __shfl_xor_sync(full, word, 1);
         word += __shfl_xor_sync(full, word, 2);
         float *const st = stage + sub * C::STRIDE;
@@ -1763,20 +1794,79 @@ __device__ __forceinline__ void fx_tile(const Record<float> *__restrict__ rec, c
     const uint32_t wend = min(wbeg + per_warp, total);
     uint32_t *s_idx = reinterpret_cast<uint32_t *>(acc + 4 * TNP);  // list_cap entries
 
+    __syncthreads();
+    constexpr int NREACH = C::R0 * C::R1 * (T2 + C::HL + C::HR);
+    const float w3 = kMaxW3<M, BLR> * 1.0001f;
+    auto bound = [&](uint32_t rowmax, uint32_t n) {  // of a node sum, in units of max |q_f|
+        return w3 * fminf(static_cast<float>(M * M) * static_cast<float>(rowmax), static_cast<float>(n));
+    };
+    uint32_t reached = total;  // particles in cells of the reach
+    if (sshift > 0 && T2 + C::HL + C::HR < ng && min(M * M * s_rowmax, total) > 256u) {
+        // Keys of several cells: the ranges hold particles below and above the reach too. Up to
+        // 256 the bound does not matter (tile_scales); above, the scale must be that of the
+        // reach. It is where the runs inside the tile alone give the same power of two (and
+        // the same answer to `dense`); otherwise the particles of the reach are counted.
+        __shared__ unsigned s_reached, s_inner, s_unsure;
+        const uint32_t outer = s_rowmax;
+        __syncthreads();
+        if (threadIdx.x == 0) s_rowmax = s_reached = s_inner = s_unsure = 0;
+        __syncthreads();
+        for (int r = threadIdx.x; r < C::R0 * C::R1; r += NT) {
+            int a0 = t0 - C::HL + r / C::R1, a1 = t1 - C::HL + r % C::R1;
+            a0 = a0 < 0 ? a0 + ng : (a0 >= ng ? a0 - ng : a0);
+            a1 = a1 < 0 ? a1 + ng : (a1 >= ng ? a1 - ng : a1);
+            const uint32_t *row = offsets + ((static_cast<int64_t>(a0) * ng + a1) * ng >> sshift);
+            const uint32_t c = row[(t2 + T2) >> sshift] - row[t2 >> sshift];
+            if (c) atomicAdd(&s_reached, c), atomicMax(&s_inner, c);
+        }
+        __syncthreads();
+        if (threadIdx.x < 4) {
+            int lo = 0, hi = 0;
+            frexpf(bound(s_inner, s_reached) * qm, &lo);
+            frexpf(bound(outer, total) * qm, &hi);
+            const bool both_dense = (s_reached > 2u * NREACH) == (total > 2u * NREACH);
+            if (lo != hi || (M == 4 && !both_dense)) atomicOr(&s_unsure, 1u);
+        }
+        __syncthreads();
+        const bool unsure = s_unsure;
+        __syncthreads();
+        if (threadIdx.x == 0) s_rowmax = unsure ? 0u : outer, s_reached = unsure ? 0u : total;
+        __syncthreads();
+        auto within = [&](uint32_t i) {
+            int d = (__float_as_int(rec[i].u.w) >> 20) - t2;
+            d = d < -C::HL ? d + ng : (d >= T2 + C::HR ? d - ng : d);
+            return d >= -C::HL && d < T2 + C::HR ? 1u : 0u;
+        };
+        for (int s0 = 0; s0 < C::MAXR && unsure; s0 += NT) {
+            const int slot = s0 + static_cast<int>(threadIdx.x);
+            const uint32_t b = slot < C::MAXR ? s_beg[slot] : 0u, len = slot < C::MAXR ? s_pre[slot + 1] - s_pre[slot] : 0u;
+            uint32_t c = 0;
+            if (len <= 8u)
+                for (uint32_t i = 0; i < len; ++i) c += within(b + i);
+            for (unsigned lng = __ballot_sync(0xffffffffu, len > 8u); lng; lng &= lng - 1u) {
+                const int l = __ffs(static_cast<int>(lng)) - 1;
+                const uint32_t lb = __shfl_sync(0xffffffffu, b, l), ln = __shfl_sync(0xffffffffu, len, l);
+                uint32_t n = 0;
+                for (uint32_t i = lane; i < ln; i += 32) n += within(lb + i);
+                n = __reduce_add_sync(0xffffffffu, n);
+                if (lane == l) c = n;
+            }
+            const uint32_t row = c + __shfl_xor_sync(0xffffffffu, c, 1);  // a row's two pieces
+            if (c) atomicAdd(&s_reached, c), atomicMax(&s_rowmax, row);
+        }
+        __syncthreads();
+        reached = s_reached;
+    }
     // dense tiles (cubic order, more than two particles per reach cell on average) sum
     // each cell's particles in registers first (cell-block path below)
-    constexpr int NREACH = C::R0 * C::R1 * (T2 + C::HL + C::HR);
-    const bool dense = M == 4 && BLR == 0 && total > 2u * NREACH && sshift == 0 && ng >= C::R0 && ng >= C::R1 &&
+    const bool dense = M == 4 && BLR == 0 && reached > 2u * NREACH && ng >= C::R0 && ng >= C::R1 &&
                        ng >= T2 + C::HL + C::HR;
     // per-field scale from order-independent bounds only (so that the grids, and the
     // spectra, do not depend on the order in which sorted particles share a cell)
-    __syncthreads();
     if (threadIdx.x < 4) {
         const int f = threadIdx.x;
         const float m = qm;  // max |q_f| over the catalogue, loaded at the start
-        const float w3 = kMaxW3<M, BLR> * 1.0001f;
-        const float reach = fminf(static_cast<float>(M * M) * static_cast<float>(s_rowmax), static_cast<float>(total));
-        tile_scales(w3 * reach * m, w3 * m, dense, s_scale[f], s_fine[f], s_shift[f]);
+        tile_scales(bound(s_rowmax, reached) * m, w3 * m, dense, s_scale[f], s_fine[f], s_shift[f]);
     }
     __syncthreads();
     const float sc0 = s_scale[0], sc1 = s_scale[1], sc2 = s_scale[2], sc3 = s_scale[3];
@@ -1801,7 +1891,7 @@ __device__ __forceinline__ void fx_tile(const Record<float> *__restrict__ rec, c
     const uint32_t chunk = min(static_cast<uint32_t>(list_cap), static_cast<uint32_t>(KP * NT));
     const bool use_list = M >= 4 || (sparse && total <= chunk);
     const bool long_rows = s_rowmax > 24u;
-    if (BLR == 0 && list_cap > 0 && use_list && !dense && sshift == 0 && ng >= C::R0 && ng >= C::R1 &&
+    if (BLR == 0 && list_cap > 0 && use_list && !dense && ng >= C::R0 && ng >= C::R1 &&
         ng >= T2 + C::HL + C::HR) {
         for (uint32_t c0 = 0; c0 < total; c0 += chunk) {
             const uint32_t cnt = min(chunk, total - c0);
@@ -1847,7 +1937,7 @@ __device__ __forceinline__ void fx_tile(const Record<float> *__restrict__ rec, c
                         const int b0 = first_node<M, C::HL, C::HR, T0>(u[k].x, packed & 1023, t0, ng);
                         const int b1 = first_node<M, C::HL, C::HR, T1>(u[k].y, (packed >> 10) & 1023, t1, ng);
                         const int b2 = first_node<M, C::HL, C::HR, T2>(u[k].z, (packed >> 20) & 1023, t2, ng);
-                        const bool reaches = M % 2 == 0 || (b0 > -M && b0 < T0 && b1 > -M && b1 < T1 && b2 > -M && b2 < T2);
+                        const bool reaches = (M % 2 == 0 && sshift == 0) || (b0 > -M && b0 < T0 && b1 > -M && b1 < T1 && b2 > -M && b2 < T2);
                         const int g = (b0 * PX + b1 * RW + b2) & 31;
                         if (reaches) key[k] = g | static_cast<int>(atomicAdd(&s_bank[g], 1u) << 5);
                     }
@@ -1901,7 +1991,7 @@ __device__ __forceinline__ void fx_tile(const Record<float> *__restrict__ rec, c
 
     if constexpr (M == 4 && BLR == 0) {  // the cell-block path uses B-spline pieces
         if (dense) {
-            deposit_cells_path<T0, T1, T2, NT>(rec, offsets, ng, t0, t1, t2, acc, TNP, PX, RW, s_fine, s_shift);
+            deposit_cells_path<T0, T1, T2, NT>(rec, offsets, ng, sshift, t0, t1, t2, acc, TNP, PX, RW, s_fine, s_shift);
             done = true;
         }
     }

@@ -177,14 +177,22 @@ AssignPlan plan_assign(const pkmom_params &p, int64_t n, int num_sms, int tile_o
     }
     int td[3];
     deposit_tile_shape(pl.tile, p.precision, td);
-    // one sort key per cell keeps each row's particles in z order, which the deposit's
-    // lane mapping relies on (coarser z segments measured slower even for sparse
-    // catalogues); segments only where 32-bit offsets would not suffice
+    // Cells per sort key (a run of cells along z). Home tiles, the direct BL stencil, FP64 and
+    // tiles of eight cells take one. Sparse FP32 gather tiles take four or two: the key table is
+    // zeroed, counted into, scanned and read back whatever the particles are (34 GB of a 1024^3
+    // assignment's traffic), and a tile only has to pass over the particles of the runs that
+    // stick out of its reach. Not beyond the density where the row bound of a tile (order^2
+    // times its fullest row's particles) usually passes 256, above which a tile has to look
+    // closer (fx_tile). 512^3 particles on 1024^3, histogram + scan + scatter + deposit: one
+    // cell a key 24.96 ms, two 23.01, four 22.42; 0.83 M on 384^3: 0.88, 0.81, 0.76.
     int sshift = 0;
-    while ((1 << (sshift + 1)) <= td[2] && (p.ng % (1 << (sshift + 1))) == 0 && cells / (1 << sshift) > double(1u << 30))
-        ++sshift;
+    if (p.precision == PKMOM_F32 && p.bl_radius == 0 && pl.tile != kHomeTile && td[2] >= 16) {
+        for (int k = 2; k > 0 && sshift == 0; --k) {
+            const double mean = ppc * (td[2] + 4.0 + (1 << k));  // particles of a row of the runs
+            if (p.order * p.order * (mean + 4.5 * std::sqrt(mean) + 2.0) <= 256.0) sshift = k;
+        }
+    }
     pl.sshift = sshift;
-    if (pl.tile == kHomeTile && sshift != 0) pl.tile = 0;  // home tiles need one sort key per cell
     // FP32 gather tiles list their particles in shared memory: room for about twice the
     // expected count of a tile's reach, at most 2048 (longer ones go 2048 at a time).
     // Orders 1 to 3 list sparse catalogues only: from half a particle per cell on, adding
