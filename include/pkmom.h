@@ -217,8 +217,10 @@ pkmom_status pkmom_estimate(pkmom_ctx *ctx, const pkmom_catalog *cat, const pkmo
 
 /* Steps 1-4 on a HOST catalogue: copies the arrays to context-owned device
  * memory (cudaMemcpyAsync; pinned host memory makes the copies asynchronous and
- * fast), runs pkmom_estimate and copies the PKMOM_NROWS * nbins result to the
- * host array out_host. Synchronises the stream before returning. */
+ * fast; the positions on the stream, velocities and masses after them on a stream of the
+ * context's own, beside the histogram and the scan), runs pkmom_estimate and copies the
+ * PKMOM_NROWS * nbins result to the host array out_host. Synchronises the stream before
+ * returning; after an error the stream's work ends with the copies. */
 pkmom_status pkmom_estimate_host(pkmom_ctx *ctx, const pkmom_catalog *cat_host, const pkmom_params *p,
                                  double *out_host, void *stream);
 
