@@ -165,10 +165,6 @@ struct SpectraTables {
     // next entry of bin_order and blocks done: [0, 2) for k_bin_shells, [2, 4) for k_bin_mu
     // (zero between launches)
     unsigned *bin_counter = nullptr;
-    // tasks of the (|k|, mu) binning and each shell's range of them (mu_task_list)
-    uint2 *mu_tasks = nullptr;
-    int *mu_range = nullptr;
-    int mu_ntasks = 0;
     size_t bytes = 0;            // device bytes of all the arrays above
 };
 cudaError_t build_spectra_tables(SpectraTables &t, int ng, int order, bool direct, int nbins, double umin,

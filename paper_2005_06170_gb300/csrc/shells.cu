@@ -45,27 +45,4 @@ std::vector<uint32_t> bin_item_list(const std::vector<int> &thresh, int ng, int 
     return work;
 }
 
-void mu_task_list(const std::vector<int> &thresh, int ng, int nbins, std::vector<uint32_t> &tasks,
-                  std::vector<int> &range)
-{
-    tasks.clear();
-    range.assign(2 * nbins, 0);
-    for (int b = nbins - 1; b >= 0; --b) {
-        range[2 * b] = range[2 * b + 1] = static_cast<int>(tasks.size() / 2);
-        const int width = thresh[b + 1] - thresh[b];
-        if (width <= 0) continue;
-        int reach = static_cast<int>(std::sqrt(static_cast<double>(thresh[b + 1] - 1)));
-        while (reach > 0 && reach * reach > thresh[b + 1] - 1) --reach;
-        while ((reach + 1) * (reach + 1) <= thresh[b + 1] - 1) ++reach;
-        reach = std::min(reach, ng / 2 - 1);
-        const int slabs = std::max(1, std::min(64, static_cast<int>(1500.0 / (1.5707963267948966 * width))));
-        for (int n0 = -reach; n0 <= reach; n0 += slabs) {
-            tasks.push_back(static_cast<uint32_t>(b));
-            tasks.push_back(static_cast<uint32_t>(n0 + ng / 2) |
-                            static_cast<uint32_t>(std::min(slabs, reach - n0 + 1)) << 16);
-        }
-        range[2 * b + 1] = static_cast<int>(tasks.size() / 2);
-    }
-}
-
 }  // namespace pkmom

@@ -23,14 +23,6 @@ int shell_tables(int nbins, double umin, double umax, std::vector<uint16_t> &bin
 // mode.
 std::vector<uint32_t> bin_item_list(const std::vector<int> &thresh, int ng, int nbins);
 
-// Tasks of the (|k|, mu) binning: runs of slabs of one shell, some 1500 modes each (a slab of
-// a shell holds about pi/2 (thresh[b+1] - thresh[b]) of them whatever its n0), the outer
-// shells first. tasks: two words each, the shell and (first n0 + ng/2) | slabs << 16, the
-// Nyquist slab left out; range: the first task of shell b and the one after its last, at 2b
-// and 2b + 1. No more tasks than (slab, shell) pairs.
-void mu_task_list(const std::vector<int> &thresh, int ng, int nbins, std::vector<uint32_t> &tasks,
-                  std::vector<int> &range);
-
 }  // namespace pkmom
 
 #endif

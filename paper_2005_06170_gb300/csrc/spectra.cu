@@ -709,8 +709,6 @@ void free_spectra_tables(SpectraTables &t)
     cudaFree(t.item_partials);
     cudaFree(t.bin_order);
     cudaFree(t.bin_counter);
-    cudaFree(t.mu_tasks);
-    cudaFree(t.mu_range);
     t = SpectraTables{};
 }
 
@@ -780,16 +778,8 @@ cudaError_t build_spectra_tables(SpectraTables &t, int ng, int order, bool direc
     if ((e = upload(reinterpret_cast<void **>(&t.bin_order), work)) != cudaSuccess) return e;
     if ((e = cudaMalloc(reinterpret_cast<void **>(&t.bin_counter), 4 * sizeof(unsigned))) != cudaSuccess) return e;
     if ((e = cudaMemset(t.bin_counter, 0, 4 * sizeof(unsigned))) != cudaSuccess) return e;
-    std::vector<uint32_t> tasks;
-    std::vector<int> range;
-    mu_task_list(thresh, ng, nbins, tasks, range);
-    t.mu_ntasks = static_cast<int>(tasks.size() / 2);
-    if (tasks.empty()) tasks.assign(2, 0);
-    if ((e = upload(reinterpret_cast<void **>(&t.mu_tasks), tasks)) != cudaSuccess) return e;
-    if ((e = upload(reinterpret_cast<void **>(&t.mu_range), range)) != cudaSuccess) return e;
     t.shell_blocks = num_sms * 4;  // resident blocks (56 registers, 256 threads)
-    t.bytes = tasks.size() * sizeof(uint32_t) + range.size() * sizeof(int) + work.size() * sizeof(uint32_t) +
-              4 * sizeof(unsigned) + bintab.size() * sizeof(uint16_t) +
+    t.bytes = work.size() * sizeof(uint32_t) + 4 * sizeof(unsigned) + bintab.size() * sizeof(uint16_t) +
               thresh.size() * sizeof(int) +
               static_cast<size_t>(ng + nh) * (prec == PKMOM_F32 ? sizeof(float) : sizeof(double)) +
               static_cast<size_t>(ng + nh) * sizeof(double) +
@@ -1321,269 +1311,20 @@ k_bin_mu(const Cx<T> *__restrict__ F, int64_t gstride, int ng, int nbins, int nm
     if (threadIdx.x == 0 && atomicAdd(counter + 1, 1u) == gridDim.x - 1) counter[0] = 0u, counter[1] = 0u;
 }
 
-// The same sums with each mode evaluated once. A warp walks the modes of a task (one shell, a
-// few slabs), finds each mode's mu bin and its mirror image's once, and queues it by bin; a
-// queue of 32 is evaluated by the 32 lanes together, summed over them by a reduce-scatter of
-// float pairs and added to the warp's totals of the bin, so that no lane idles whatever the
-// order of the bins and no mode is visited once per bin. Queues 0 .. nmu-1 hold the modes
-// whose mirror image (the mode -n, where l > 0) falls in the mirrored bin nmu-1-m: their sums
-// are added to both. Queues nmu .. 2 nmu-1 hold the others (l = 0, or a mirror image in
-// another bin, as on a bin's edge), once per bin, with a sign for the odd terms. Bound by
-// issue; visiting every mode once per bin took eight times the instructions at nmu = 8
-// (256^3, 32 x 8 cells: 0.47 ms for the stage, see k_reduce_finalize_mu for the rest).
-// bins the queues serve: eight warps' queues and totals (1.2 or 2.4 KB a bin and warp) have to
-// fit one SM's shared memory; more bins take k_bin_mu
-template <typename T> constexpr int kMuQueueMax = sizeof(T) == 4 ? 16 : 8;
-constexpr int kMuQueue = 64;      // entries of a queue: 31 left over and 32 new
-constexpr int kMuPad = 24;        // kMuVals padded to whole reduce-scatters
-template <typename T> struct MuEntry { uint32_t at; T h; };  // i0 | i1 << 10 | l << 20, sign in bit 31; row's h
-template <typename T>
-__host__ __device__ constexpr size_t mu_warp_bytes(int nmu)
-{
-    return size_t(nmu) * (2 * kMuQueue * sizeof(MuEntry<T>) + 2 * kMuPad * sizeof(T) + 2 * sizeof(int));
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kBinThreads, 2)
-k_bin_mu_queue(const Cx<T> *__restrict__ F, int64_t gstride, int ng, int nmu, const int *__restrict__ thresh,
-               const T *__restrict__ gf, const T *__restrict__ gh, const double *__restrict__ hf,
-               const double *__restrict__ hh, const double *__restrict__ mom, double ge0, double ge1, double ge2,
-               int bulk_dir, const uint2 *__restrict__ tasks, int ntasks, unsigned *__restrict__ counter,
-               double *__restrict__ partials)
-{
-    constexpr int NW = kBinThreads / 32;
-    constexpr unsigned full = 0xffffffffu;
-    extern __shared__ __align__(16) unsigned char mu_smem[];
-    __shared__ int4 s_rows[NW][32];
-    __shared__ T s_rowh[NW][32];
-    __shared__ double s_dir[9];  // v_b, its direction, the binning direction
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nh = ng / 2 + 1;
-    T *s_hh = reinterpret_cast<T *>(mu_smem);
-    unsigned char *own = mu_smem + (size_t(nh) * sizeof(T) + 15) / 16 * 16 + size_t(w) * ((mu_warp_bytes<T>(nmu) + 15) / 16 * 16);
-    auto *queue = reinterpret_cast<MuEntry<T> *>(own);                        // [2 nmu][kMuQueue]
-    T *tot_hi = reinterpret_cast<T *>(queue + 2 * nmu * kMuQueue), *tot_lo = tot_hi + nmu * kMuPad;
-    int *fill = reinterpret_cast<int *>(tot_lo + nmu * kMuPad);               // [2 nmu]
-    for (int k = threadIdx.x; k < nh; k += kBinThreads) s_hh[k] = static_cast<T>(hh[k]);
-    if (threadIdx.x < 3) s_dir[threadIdx.x] = mom[2 + threadIdx.x] / mom[0];
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        const double vbn = sqrt(s_dir[0] * s_dir[0] + s_dir[1] * s_dir[1] + s_dir[2] * s_dir[2]);
-        const double eb = vbn > 0 ? s_dir[threadIdx.x] / vbn : 0.0;
-        s_dir[3 + threadIdx.x] = eb;
-        s_dir[6 + threadIdx.x] = bulk_dir ? eb : threadIdx.x == 0 ? ge0 : threadIdx.x == 1 ? ge1 : ge2;
-    }
-    __syncthreads();
-    const T vb0 = static_cast<T>(s_dir[0]), vb1 = static_cast<T>(s_dir[1]), vb2 = static_cast<T>(s_dir[2]);
-    const T eb0 = static_cast<T>(s_dir[3]), eb1 = static_cast<T>(s_dir[4]), eb2 = static_cast<T>(s_dir[5]);
-    // the bin decision in FP32; the mean mu in the grid precision
-    const float e0 = static_cast<float>(s_dir[6]), e1 = static_cast<float>(s_dir[7]), e2 = static_cast<float>(s_dir[8]);
-    const T et0 = static_cast<T>(s_dir[6]), et1 = static_cast<T>(s_dir[7]), et2 = static_cast<T>(s_dir[8]);
-    for (int k = lane; k < 2 * nmu * kMuPad; k += 32) tot_hi[k] = T(0);
-    for (int k = lane; k < 2 * nmu; k += 32) fill[k] = 0;
-    __syncwarp();
-
-    // evaluates the first n entries of queue `key` and adds their sums to the totals
-    auto flush = [&](int key, int n) {
-        const bool both = key < nmu;
-        const int m = both ? key : key - nmu;
-        T v[kMuPad];
-#pragma unroll
-        for (int k = 0; k < kMuPad; ++k) v[k] = T(0);
-        if (lane < n) {
-            const MuEntry<T> en = queue[key * kMuQueue + lane];
-            const int i0 = en.at & 1023, i1 = (en.at >> 10) & 1023, l = (en.at >> 20) & 1023;
-            const int n0 = i0 < ng / 2 ? i0 : i0 - ng, nn1 = i1 < ng / 2 ? i1 : i1 - ng;
-            const int64_t mi = (static_cast<int64_t>(i0) * ng + i1) * nh + l;
-            if (PK_IN(mi, gstride, kChkMode) && PK_IN(l, nh, kChkMode)) {
-                const T g = gf[i0] * gf[i1] * gh[l];
-                const T th = en.h * s_hh[l];
-                const Cx<T> dd = F[mi], p0 = F[gstride + mi], p1 = F[2 * gstride + mi], p2 = F[3 * gstride + mi];
-                const int nsq = n0 * n0 + nn1 * nn1 + l * l;
-                const T a0 = static_cast<T>(n0), a1 = static_cast<T>(nn1), a2 = static_cast<T>(l);
-                const T kr = a0 * p0.x + a1 * p1.x + a2 * p2.x, ki = a0 * p0.y + a1 * p1.y + a2 * p2.y;
-                const Cx<T> q0{p0.x - vb0 * dd.x, p0.y - vb0 * dd.y};
-                const Cx<T> q1{p1.x - vb1 * dd.x, p1.y - vb1 * dd.y};
-                const Cx<T> q2{p2.x - vb2 * dd.x, p2.y - vb2 * dd.y};
-                const T jr = a0 * q0.x + a1 * q1.x + a2 * q2.x, ji = a0 * q0.y + a1 * q1.y + a2 * q2.y;
-                const T br = eb0 * q0.x + eb1 * q1.x + eb2 * q2.x, bi = eb0 * q0.y + eb1 * q1.y + eb2 * q2.y;
-                v[0] = g * (dd.x * dd.x + dd.y * dd.y);
-                v[1] = g * (p0.x * p0.x + p0.y * p0.y + p1.x * p1.x + p1.y * p1.y + p2.x * p2.x + p2.y * p2.y);
-                v[2] = g * (q0.x * q0.x + q0.y * q0.y + q1.x * q1.x + q1.y * q1.y + q2.x * q2.x + q2.y * q2.y);
-                v[3] = g * (kr * kr + ki * ki);
-                v[4] = g * (jr * jr + ji * ji);
-                v[5] = g * (dd.x * ki - dd.y * kr);  // Im(conj(F_d) n.F_p)
-                v[6] = g * (dd.x * kr + dd.y * ki);  // Re(conj(F_d) n.F_p)
-                v[7] = g * (dd.x * ji - dd.y * jr);
-                v[8] = g * (dd.x * jr + dd.y * ji);
-                v[9] = g * (dd.x * br + dd.y * bi);
-                const T rt = sqrt(static_cast<T>(nsq));
-                v[10] = T(1);
-                v[11] = rt;
-                v[12] = (a0 * et0 + a1 * et1 + a2 * et2) / rt;
-                v[13] = th;
-                v[14] = th * a0 * a0;
-                v[15] = th * a1 * a1;
-                v[16] = th * a2 * a2;
-                v[17] = th * a0 * a1;
-                v[18] = th * a0 * a2;
-                v[19] = th * a1 * a2;
-                v[20] = th * a0;
-                v[21] = th * a1;
-                v[22] = th * a2;
-                if (en.at >> 31) {
-#pragma unroll
-                    for (int k = 0; k < kMuVals; ++k)
-                        if (mu_odd(k)) v[k] = -v[k];
-                }
-            }
-        }
-        // lane 4j + c holds the sum of value 8g + j: c = 0 adds it to bin m, c = 1 to the mirror
-        const int c = lane & 3, bin = c == 0 ? m : nmu - 1 - m;
-#pragma unroll
-        for (int g = 0; g < kMuPad / 8; ++g) {
-            T hi[8], lo[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) hi[k] = v[8 * g + k], lo[k] = T(0);
-            warp_scatter_pair8(hi, lo);
-            const int k = 8 * g + (lane >> 2);
-            const int at = bin * kMuPad + k;
-            const bool neg = c == 1 && mu_odd(k);
-            // in turn: for nmu odd, the middle bin is its own mirror
-            for (int turn = 0; turn < (both ? 2 : 1); ++turn) {
-                if (c == turn) {
-                    T th = tot_hi[at], tl = tot_lo[at];
-                    pair_add(th, tl, neg ? -hi[0] : hi[0], neg ? -lo[0] : lo[0]);
-                    tot_hi[at] = th, tot_lo[at] = tl;
-                }
-                __syncwarp();
-            }
-        }
-    };
-    // queues the lanes' entries (push: this lane has one) and evaluates the queues that fill
-    auto push = [&](bool has, int key, uint32_t at, T h) {
-        const unsigned who = __ballot_sync(full, has);
-        if (!who) return;
-        const unsigned same = __match_any_sync(full, has ? key : -1 - lane);
-        int n = 0;
-        if (has) {
-            n = fill[key];
-            queue[key * kMuQueue + n + __popc(same & ((1u << lane) - 1u))] = MuEntry<T>{at, h};
-            n += __popc(same);
-        }
-        __syncwarp();
-        const bool lead = has && __ffs(static_cast<int>(same)) - 1 == lane;
-        if (lead) fill[key] = n >= 32 ? n - 32 : n;
-        for (unsigned ready = __ballot_sync(full, lead && n >= 32); ready; ready &= ready - 1u) {
-            const int src = __ffs(static_cast<int>(ready)) - 1;
-            const int fk = __shfl_sync(full, key, src), left = __shfl_sync(full, n, src) - 32;
-            flush(fk, 32);
-            MuEntry<T> mv{};
-            if (lane < left) mv = queue[fk * kMuQueue + 32 + lane];
-            __syncwarp();
-            if (lane < left) queue[fk * kMuQueue + lane] = mv;
-            __syncwarp();
-        }
-        __syncwarp();
-    };
-
-    for (;;) {
-        unsigned jt = 0;
-        if (lane == 0) jt = atomicAdd(counter, 1u);
-        jt = __shfl_sync(full, jt, 0);
-        if (jt >= static_cast<unsigned>(ntasks)) break;
-        const uint2 task = tasks[jt];  // shell; first n0 + ng/2 and the number of slabs
-        const int b = static_cast<int>(task.x), first = static_cast<int>(task.y & 0xffff) - ng / 2,
-                  slabs = static_cast<int>(task.y >> 16);
-        const int lo2 = thresh[b], hi2 = thresh[b + 1];  // lo2 <= |n|^2 < hi2
-        for (int n0 = first; n0 < first + slabs; ++n0) {
-            const int i0 = n0 < 0 ? n0 + ng : n0;
-            const int rem = hi2 - 1 - n0 * n0;
-            if (n0 == -ng / 2 || hi2 <= lo2 || rem < 0) continue;
-            const int R1 = isqrt_floor(rem);
-            const int n1lo = max(1 - ng / 2, -R1), n1hi = min(ng / 2 - 1, R1);
-            const double h0 = hf[i0];
-            for (int r0 = n1lo; r0 <= n1hi; r0 += 32) {
-                const int n1 = r0 + lane;
-                const bool row = n1 <= n1hi;
-                int l_lo = 0, len = 0;
-                if (row) {
-                    const int r2 = n0 * n0 + n1 * n1;
-                    const int top = hi2 - 1 - r2;
-                    if (top >= 0) {
-                        const int lh = min(isqrt_floor(top), nh - 2);  // no Nyquist plane
-                        const int need = lo2 - r2;
-                        const int ll = need <= 0 ? 0 : isqrt_floor(need - 1) + 1;
-                        if (lh >= ll) l_lo = ll, len = lh - ll + 1;
-                    }
-                }
-                int inc = len;
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const int t = __shfl_up_sync(full, inc, d);
-                    if (lane >= d) inc += t;
-                }
-                const int total = __shfl_sync(full, inc, 31);
-                if (total == 0) continue;
-                const int pre = inc - len;
-                const unsigned nonempty = __ballot_sync(full, len > 0);
-                if (len > 0) {  // compacted: the k-th non-empty row at index k
-                    const int i1 = n1 < 0 ? n1 + ng : n1, at = __popc(nonempty & ((1u << lane) - 1u));
-                    s_rows[w][at] = make_int4(pre, l_lo, n1, i1);
-                    s_rowh[w][at] = static_cast<T>(h0 * hf[i1]);
-                }
-                __syncwarp();
-                for (int w0 = 0; w0 < total; w0 += 32) {
-                    // the row of mode w0 + lane: the last one starting at or before it
-                    const bool in_win = len > 0 && pre >= w0 && pre < w0 + 32;
-                    const unsigned starts = __reduce_or_sync(full, in_win ? 1u << (pre - w0) : 0u);
-                    const int before = __popc(__ballot_sync(full, len > 0 && pre < w0));
-                    const bool ok = w0 + lane < total;
-                    const int q = before + __popc(starts & (full >> (31 - lane))) - 1;
-                    const int4 rw = s_rows[w][ok ? q : 0];
-                    const T rowh = s_rowh[w][ok ? q : 0];
-                    const int l = ok ? rw.y + (w0 + lane - rw.x) : 0, nn1 = rw.z;
-                    const float rn = __fsqrt_rn(static_cast<float>(n0 * n0 + nn1 * nn1 + l * l));
-                    const int mf = mu_bin(static_cast<float>(n0), static_cast<float>(nn1), static_cast<float>(l), e0, e1, e2, rn, nmu);
-                    const int mr = mu_bin(-static_cast<float>(n0), -static_cast<float>(nn1), -static_cast<float>(l), e0, e1, e2, rn, nmu);
-                    const bool regular = l > 0 && mr == nmu - 1 - mf;
-                    const uint32_t at = static_cast<uint32_t>(i0) | static_cast<uint32_t>(rw.w) << 10 | static_cast<uint32_t>(l) << 20;
-                    push(ok, regular ? mf : nmu + mf, at, rowh);
-                    push(ok && l > 0 && !regular, nmu + mr, at | 1u << 31, rowh);  // the mirror image on its own
-                }
-                __syncwarp();
-            }
-        }
-        for (int key = 0; key < 2 * nmu; ++key) {  // what is left of the task
-            const int n = fill[key];
-            if (n) flush(key, n);
-        }
-        __syncwarp();
-        double *out = partials + static_cast<int64_t>(jt) * nmu * kMuVals;
-        for (int k = lane; k < nmu * kMuVals; k += 32) {
-            const int at = (k / kMuVals) * kMuPad + k % kMuVals;
-            out[k] = static_cast<double>(tot_hi[at]) + static_cast<double>(tot_lo[at]);
-        }
-        __syncwarp();
-        for (int k = lane; k < 2 * nmu * kMuPad; k += 32) tot_hi[k] = T(0);
-        for (int k = lane; k < 2 * nmu; k += 32) fill[k] = 0;
-        __syncwarp();
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(counter + 1, 1u) == gridDim.x - 1) counter[0] = 0u, counter[1] = 0u;
-}
-
 struct MuParams {
     double V, kf, ts;
     int ncells;
 };
 
-// The sums of a (shell, mu) cell -> spectra with the shot noise
+// One thread per (shell, mu) cell: the sums of k_bin_mu -> spectra with the shot noise
 // subtracted in FP64 (the same algebra as k_finalize, with the odd terms kept).
-template <class Sums>
-__device__ __forceinline__ void finalize_mu(Sums S, int cidx, const double *__restrict__ mom, const MuParams &fp,
-                                            double *__restrict__ out /*[PKMOM_MU_NROWS][ncells]*/)
+__global__ void k_finalize_mu(const double *__restrict__ sums /*[kMuVals][ncells]*/, const double *__restrict__ mom,
+                              MuParams fp, double *__restrict__ out /*[PKMOM_MU_NROWS][ncells]*/)
 {
+    const int cidx = blockIdx.x * blockDim.x + threadIdx.x;
     const int nc = fp.ncells;
+    if (cidx >= nc) return;
+    auto S = [&](int k) { return sums[k * nc + cidx]; };
     auto put = [&](int row, double v) { out[row * nc + cidx] = v; };
     const double n = S(10);
     put(PKMOM_MU_ROW_NMODES, n);
@@ -1632,33 +1373,6 @@ __device__ __forceinline__ void finalize_mu(Sums S, int cidx, const double *__re
     put(PKMOM_MU_ROW_IM_DT_B, -cx * S(8) - im_sn_b);
     put(PKMOM_MU_ROW_RE_DPB_B, c * (S(9) - ebR * H));
 }
-__global__ void k_finalize_mu(const double *__restrict__ sums /*[kMuVals][ncells]*/, const double *__restrict__ mom,
-                              MuParams fp, double *__restrict__ out)
-{
-    const int cidx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cidx < fp.ncells) finalize_mu([&](int k) { return sums[k * fp.ncells + cidx]; }, cidx, mom, fp, out);
-}
-
-// One block per (shell, mu) cell: the partials of the shell's tasks (range[2 shell] ..
-// range[2 shell + 1] - 1) added in a fixed order, then the cell's rows.
-__global__ void __launch_bounds__(128)
-k_reduce_finalize_mu(const double *__restrict__ partials, const int *__restrict__ range, int nmu,
-                     const double *__restrict__ mom, MuParams fp, double *__restrict__ out)
-{
-    __shared__ double s_sum[4][kMuVals];
-    const int b = blockIdx.x / nmu, m = blockIdx.x % nmu, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane < kMuVals) {
-        double x = 0.0;
-        for (int t = range[2 * b] + w; t < range[2 * b + 1]; t += 4)
-            x += partials[(static_cast<int64_t>(t) * nmu + m) * kMuVals + lane];
-        s_sum[w][lane] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x < kMuVals)
-        s_sum[0][threadIdx.x] = (s_sum[0][threadIdx.x] + s_sum[1][threadIdx.x]) + (s_sum[2][threadIdx.x] + s_sum[3][threadIdx.x]);
-    __syncthreads();
-    if (threadIdx.x == 0) finalize_mu([&](int k) { return s_sum[0][k]; }, blockIdx.x, mom, fp, out);
-}
 
 }  // namespace
 
@@ -1671,33 +1385,6 @@ cudaError_t launch_spectra_mu(const SpectraTables &t, const pkmom_params &p, con
     const unsigned blocks = static_cast<unsigned>(t.shell_blocks) / 2u;  // resident: 2 blocks per SM
     const double d0 = dir ? dir[0] : 0.0, d1 = dir ? dir[1] : 0.0, d2 = dir ? dir[2] : 0.0;
     const int bulk_dir = dir ? 0 : 1;
-    MuParams fp;
-    fp.V = p.box_L * p.box_L * p.box_L;
-    fp.kf = kTwoPi / p.box_L;
-    fp.ts = p.theta_scale;
-    fp.ncells = t.nbins * nmu;
-    if (nmu <= (t.prec == PKMOM_F32 ? kMuQueueMax<float> : kMuQueueMax<double>)) {
-        auto launch = [&](auto kern, auto zero) -> cudaError_t {
-            using T = decltype(zero);
-            const size_t smem = (size_t(nh) * sizeof(T) + 15) / 16 * 16 +
-                                (kBinThreads / 32) * ((mu_warp_bytes<T>(nmu) + 15) / 16 * 16);
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-            if (e != cudaSuccess) return e;
-            const unsigned nblk = static_cast<unsigned>(
-                std::min<int64_t>(blocks, (t.mu_ntasks + kBinThreads / 32 - 1) / (kBinThreads / 32)));
-            if (nblk)
-                kern<<<nblk, kBinThreads, smem, s>>>(static_cast<const Cx<T> *>(grids), gstride, ng, nmu, t.thresh,
-                                                     static_cast<const T *>(t.g_full), static_cast<const T *>(t.g_half),
-                                                     t.h_full, t.h_half, moments_dev, d0, d1, d2, bulk_dir, t.mu_tasks,
-                                                     t.mu_ntasks, t.bin_counter + 2, partials);
-            return cudaGetLastError();
-        };
-        const cudaError_t e = t.prec == PKMOM_F32 ? launch(k_bin_mu_queue<float>, 0.0f) : launch(k_bin_mu_queue<double>, 0.0);
-        if (e != cudaSuccess) return e;
-        k_reduce_finalize_mu<<<fp.ncells, 128, 0, s>>>(partials, t.mu_range, nmu, moments_dev, fp, out);
-        st.launches += 2;
-        return cudaGetLastError();
-    }
     if (t.prec == PKMOM_F32)
         k_bin_mu<float><<<blocks, kBinThreads, 0, s>>>(
             static_cast<const Cx<float> *>(grids), gstride, ng, t.nbins, nmu, t.thresh,
@@ -1708,8 +1395,13 @@ cudaError_t launch_spectra_mu(const SpectraTables &t, const pkmom_params &p, con
             static_cast<const Cx<double> *>(grids), gstride, ng, t.nbins, nmu, t.thresh,
             static_cast<const double *>(t.g_full), static_cast<const double *>(t.g_half), t.h_full, t.h_half,
             moments_dev, d0, d1, d2, bulk_dir, t.bin_order, t.bin_nwork, t.bin_counter + 2, partials);
-    const int ncells = fp.ncells;
+    const int ncells = t.nbins * nmu;
     k_reduce_items<kMuVals><<<ncells, 256, 0, s>>>(partials, ng, ncells, sums, t.thresh, nmu);
+    MuParams fp;
+    fp.V = p.box_L * p.box_L * p.box_L;
+    fp.kf = kTwoPi / p.box_L;
+    fp.ts = p.theta_scale;
+    fp.ncells = ncells;
     k_finalize_mu<<<(ncells + 127) / 128, 128, 0, s>>>(sums, moments_dev, fp, out);
     st.launches += 3;
     return cudaGetLastError();

@@ -30,7 +30,7 @@ __device__ __forceinline__ void pair_add(double &hi, double &lo, double bh, doub
 // same in lanes 4k..4k+3; 9 pair additions per lane instead of 40 for eight butterflies.
 // Returned as FP64; fixed order.
 template <typename T>
-__device__ __forceinline__ void warp_scatter_pair8(T (&hi)[8], T (&lo)[8])  // the sum in hi[0] + lo[0]
+__device__ __forceinline__ double warp_scatter_sum8(T (&hi)[8], T (&lo)[8])
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -51,11 +51,6 @@ __device__ __forceinline__ void warp_scatter_pair8(T (&hi)[8], T (&lo)[8])  // t
         const T rh = __shfl_xor_sync(full, hi[0], o), rl = __shfl_xor_sync(full, lo[0], o);
         pair_add(hi[0], lo[0], rh, rl);
     }
-}
-template <typename T>
-__device__ __forceinline__ double warp_scatter_sum8(T (&hi)[8], T (&lo)[8])
-{
-    warp_scatter_pair8(hi, lo);
     return static_cast<double>(hi[0]) + static_cast<double>(lo[0]);
 }
 
