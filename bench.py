@@ -59,24 +59,24 @@ DEFAULT = "zeldovich512_ng512"
 # capture of the current kernels; a stage whose kernels change drops its entry until
 # it is captured again
 MEASURED_TRAFFIC = {
-    ("zeldovich512_ng512", "deposit"): ((4981.8 + 3626.1 + 3716.0 + 1623.8) * 1e6,
+    ("zeldovich512_ng512", "deposit"): (8 * (630.6 + 416.6 + 457.8 + 168.7) * 1e6,
                                         "ncu dram__bytes_read.sum + dram__bytes_write.sum of k_deposit_home and "
-                                        "k_home_fixup, mean of 5 launches of the 512^3 workload "
-                                        "(profiles/launches_zeldovich512_ng512.md)"),
+                                        "k_home_fixup, one launch of each at 256^3 particles on 256^3 "
+                                        "(profiles/own_kernels.md), times 8"),
     # the same density (1/8 particle per cell) captured at 256^3 particles on 512^3 and
     # scaled by 8: the records read, the key rows read and the grid written all grow with
     # the particles and cells, which are both 8 times as many
-    ("zeldovich512_ng1024", "deposit"): (8 * (1.27 + 2.11) * 1e9,
+    ("zeldovich512_ng1024", "deposit"): (8 * (0.766 + 2.105) * 1e9,
                                          "ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_deposit_fx "
                                          "launch on 256^3 particles and a 512^3 grid "
-                                         "(profiles/deposit_sparse_zeldovich256_ng512.md), times 8"),
+                                         "(profiles/own_kernels.md), times 8"),
 }
 # warp instructions per launch of the dominant kernel, from one ncu --set full capture of
 # the current kernel on the 256^3 workload, scaled to other workloads by particle count
 # (the same work per particle at one particle per cell)
 MEASURED_INSTRUCTIONS = {
-    "k_deposit_home": (596.13e6, 256 ** 3, "ncu smsp__inst_executed.sum of k_deposit_home on the 256^3 workload "
-                                         "(profiles/kernels_zeldovich256_ng256.md), scaled by particles"),
+    "k_deposit_home": (544.75e6, 256 ** 3, "ncu smsp__inst_executed.sum of k_deposit_home, 256^3 Zel'dovich "
+                                         "particles on 256^3 (profiles/own_kernels.md), scaled by particles"),
 }
 # configs 4 and 5 run through their own drivers below
 MULTI = {
@@ -359,7 +359,7 @@ def bin_roofline(stage_ms, ng, prec):
     b = 4 * 2 * elem * in_shell_modes(ng)
     ms = stage_ms["bin"]
     gbs = b / (ms * 1e-3) / 1e9 if ms > 0 else None
-    return {"kernel": "k_bin_shells + k_reduce_items", "bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s",
+    return {"kernel": "k_bin_shells + k_reduce_finalize", "bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s",
             "frac": gbs / peak if gbs else None, "algorithmic_bytes_per_launch": b, "avg_launch_ms": ms,
             "bytes_16B_per_cell": full, "frac_16B_per_cell": full / (ms * 1e-3) / 1e9 / peak if ms > 0 else None}
 

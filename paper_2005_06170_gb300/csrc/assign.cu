@@ -12,7 +12,8 @@
 //   k_moments       FP64 moments and max |q|, from velocities and masses.
 //   k_deposit_home  (FP32, cubic, >= 1/2 particle per cell) each particle deposited
 //   + k_home_fixup  once by the tile owning its cell, halos added afterwards; otherwise
-//   k_deposit(_fx)  one CTA per output tile gathers the particles of every segment whose
+//   k_deposit_fx    (FP32), k_deposit_ix (FP64, orders 2 to 5, in integers), k_deposit
+//                   (FP64, the rest): one CTA per output tile gathers the particles of every segment whose
 //                   stencils reach the tile, accumulates in shared memory, then writes
 //                   each node of the tile exactly once. No global atomics, no zero fill.
 #include <algorithm>
@@ -2154,7 +2155,8 @@ k_deposit_fx_batch(const FxBatch jobs, unsigned long long *__restrict__ counter)
 // deposited 32 at a time, one per lane. Bound by the shared pipe and by latency together
 // (shared memory holds two tiles per SM). Two cells a lane instead of four add 5 node sums
 // for 2 cells instead of 7 for 4, but fit 80 registers instead of 128, so that 24 warps run
-// on an SM instead of 16: 512^3 particles on 512^3, deposit 8.99 -> 8.75 ms.
+// on an SM instead of 16: 512^3 particles on 512^3, deposit 8.99 -> 8.75 ms,
+// and with the dy loop of home_pair unrolled and one queue of extra particles 8.04 ms.
 // Tiles with more than two particles per cell, or 32 in some four consecutive cells of a
 // column, take the cell-block path: one warp per cell, each contribution rounded at the
 // fine scale (largest contribution < 2^22) and summed exactly, in 64-bit shared

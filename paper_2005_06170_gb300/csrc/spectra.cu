@@ -188,7 +188,7 @@ __device__ __forceinline__ int isqrt_floor(int x)
 // and consecutive lanes read consecutive modes of a row. The seven per-mode
 // values are summed with Kahan-compensated adds in the grid precision; one warp
 // reduce-scatter per item (float pairs for FP32) writes partials[item][kBinVals] in FP64,
-// and k_reduce_items adds the items of each shell in a fixed order.
+// and k_reduce_finalize adds the items of each shell in a fixed order.
 // Per-warp staging of the rows of one item (k_bin_shells, k_bin_batch): the non-empty
 // rows of a group of 32, in order, each as (first mode's index in the joined list, first
 // l, n1, then for FP32 the bits of the row's factor g0 * gf[i1], for FP64 i1), one
