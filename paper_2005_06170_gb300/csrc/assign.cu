@@ -1366,8 +1366,10 @@ struct FxLayout {
     }
 };
 
-// Every node the listed path adds to (weights of nodes outside the tile zero) lies in the
-// padded allocation: node coordinates run from -HL + first(0) to (T + HR - 1) + first(1/2)
+// Every node the listed paths add to (weights of nodes outside the tile zero) lies in the
+// padded allocation, for particles of cells within reach of the tile, or for which the reach
+// test of the list holds (with keys of several cells the runs hold others too, whose
+// coordinates can be off by ng: the list and coop_deposit leave those out): node coordinates run from -HL + first(0) to (T + HR - 1) + first(1/2)
 // + M - 1 on each axis (first is smallest at t = 0 and largest from t = 1/2 on).
 template <int M, int T0, int T1, int T2>
 constexpr bool fx_pads_cover()
@@ -1718,7 +1720,7 @@ __device__ __forceinline__ void coop_deposit(const Record<float> *__restrict__ r
 // nearest even, one rounding of the exact product). The bound depends only on counts
 // and maxima, and integer sums do not depend on order: the grids are the same whatever
 // order the sort leaves particles of one cell in.
-constexpr int kListRankMax = 128;  // largest bank group whose list entries are reordered
+constexpr int kListRankMax = 128;  // ranks within a bank group that the list is ordered by
 
 // One tile of the FP32 gather deposit (the body of k_deposit_fx, and of each work item
 // of its persistent batched form k_deposit_fx_batch). The whole CTA takes part; its
@@ -1957,25 +1959,37 @@ __device__ __forceinline__ void fx_tile(const Record<float> *__restrict__ rec, c
                     continue;
                 }
             }
-            uint32_t len = cnt;
-            if (maxc <= static_cast<uint32_t>(kListRankMax)) {
-                // entries before (r, g): sum over groups of min(count, r), then the groups
-                // below g with more than r entries
-                for (uint32_t r = warp; r < maxc; r += NW) {
-                    const unsigned m = __ballot_sync(0xffffffffu, bank > r);
-                    const uint32_t below = __reduce_add_sync(0xffffffffu, bank < r ? bank : r);
-                    if (lane == 0) s_rmask[r] = m, s_rbase[r] = below;
-                }
-                len = __reduce_add_sync(0xffffffffu, bank);
-                __syncthreads();
-#pragma unroll
-                for (int k = 0; k < KP; ++k) {
-                    if (key[k] < 0) continue;
-                    const int g = key[k] & 31, r = key[k] >> 5;
-                    s_idx[s_rbase[r] + __popc(s_rmask[r] & ((1u << g) - 1u))] = idx[k];
-                }
-                __syncthreads();
+            // Only particles that reach the tile go to banked_particle (the pads cover no others):
+            // entries before (r, g): sum over groups of min(count, r), then the groups below g
+            // with more than r entries; ranks from kListRankMax on come last, group by group
+            constexpr uint32_t kRanks = kListRankMax;
+            for (uint32_t r = warp; r < min(maxc, kRanks); r += NW) {
+                const unsigned m = __ballot_sync(0xffffffffu, bank > r);
+                const uint32_t below = __reduce_add_sync(0xffffffffu, bank < r ? bank : r);
+                if (lane == 0) s_rmask[r] = m, s_rbase[r] = below;
             }
+            const uint32_t len = __reduce_add_sync(0xffffffffu, bank);
+            uint32_t last = 0;  // lane g: the place of group g's entry of rank kListRankMax
+            if (maxc > kRanks) {
+                const uint32_t over = bank > kRanks ? bank - kRanks : 0u;
+                uint32_t upto = over;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t x = __shfl_up_sync(0xffffffffu, upto, o);
+                    if (lane >= o) upto += x;
+                }
+                last = __reduce_add_sync(0xffffffffu, min(bank, kRanks)) + upto - over;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < KP; ++k) {
+                const int g = key[k] & 31, r = key[k] >> 5;
+                const uint32_t from = __shfl_sync(0xffffffffu, last, g);
+                if (key[k] < 0) continue;
+                s_idx[r < kListRankMax ? s_rbase[r] + __popc(s_rmask[r] & ((1u << g) - 1u)) : from + r - kListRankMax] =
+                    idx[k];
+            }
+            __syncthreads();
             const unsigned acc_s = static_cast<unsigned>(__cvta_generic_to_shared(acc));
             uint32_t p = threadIdx.x;  // warp w takes chunks w, w + NW, ... of 32 entries
             Record<float> nxt;
