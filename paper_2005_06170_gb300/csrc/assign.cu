@@ -1449,6 +1449,17 @@ __device__ __forceinline__ int first_node(float t, int cell, int corner, int ng)
     return d + bspline_first<M, float>(t);
 }
 
+// A value on the tile's scale for the listed paths, which add value times weight to nodes
+// outside the tile too, relying on weight zero: NaN and infinities, whose product with zero is
+// not zero, become the largest value of the scale (finite values are below it: tile_scales).
+// Without this a NaN velocity changed other nodes and list entries, that is, record indices.
+template <int M>
+__device__ __forceinline__ float listed_value(float q, float scale)
+{
+    constexpr float top = 4194304.0f / kMaxWeight3<M>;  // weights times value below 2^22
+    return fminf(fmaxf(q * scale, -top), top);
+}
+
 // One particle of the reordered list (see k_deposit_fx): its M^3 stencil nodes at
 // immediate offsets from the shared-window address of its first node, with the weights of
 // nodes outside the tile set to zero (no branch or predicate per node; see FxLayout). The
@@ -1485,7 +1496,8 @@ __device__ __forceinline__ void banked_particle(const Record<float> &r, int ng, 
         !PK_IN(b2 - LO, T2 + HI - LO + 1, kChkShared))
         return;
     const unsigned base = acc_s + 4u * static_cast<unsigned>(b0 * PX + b1 * RW + b2);
-    const float qs[4] = {r.q.x * sc0, r.q.y * sc1, r.q.z * sc2, r.q.w * sc3};
+    const float qs[4] = {listed_value<M>(r.q.x, sc0), listed_value<M>(r.q.y, sc1), listed_value<M>(r.q.z, sc2),
+                         listed_value<M>(r.q.w, sc3)};
     f32x2 qp[4], zp[(M + 1) / 2];  // each value twice, the z weights in pairs (fma.rn.f32x2)
 #pragma unroll
     for (int f = 0; f < 4; ++f) qp[f] = f2_pack(qs[f], qs[f]);
@@ -1640,11 +1652,13 @@ __device__ __forceinline__ void coop_deposit(const Record<float> *__restrict__ r
             } else {
                 const float wf = __int_as_float(word);
                 float4 *o = reinterpret_cast<float4 *>(st + C::QW);
+                const float4 qs = make_float4(listed_value<M>(q.x, sc0), listed_value<M>(q.y, sc1),
+                                              listed_value<M>(q.z, sc2), listed_value<M>(q.w, sc3));
                 if constexpr (M == 4) {
-                    o[0] = make_float4(q.x * sc0, q.y * sc1, wf, 0.f);
-                    o[1] = make_float4(q.z * sc2, q.w * sc3, wf, 0.f);
+                    o[0] = make_float4(qs.x, qs.y, wf, 0.f);
+                    o[1] = make_float4(qs.z, qs.w, wf, 0.f);
                 } else {
-                    o[0] = make_float4(q.x * sc0, q.y * sc1, q.z * sc2, q.w * sc3);
+                    o[0] = qs;
                     st[C::QW + 4] = wf;
                 }
             }
