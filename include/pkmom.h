@@ -178,7 +178,13 @@ size_t pkmom_footprint_bytes(const pkmom_params *p, int64_t n);
  * grids at `grids` (pkmom_grid_bytes bytes, device, 16-byte aligned; every real
  * element is written, the two padding elements of each row are not). `scratch` is
  * 16-byte aligned device memory of at least pkmom_assign_scratch_bytes bytes (else
- * PKMOM_ESCRATCH). Misaligned grids or scratch give PKMOM_EINVAL. */
+ * PKMOM_ESCRATCH). Misaligned grids or scratch give PKMOM_EINVAL.
+ *
+ * Rounding of the grids. FP32: each contribution to one step of a tile's fixed-point scale
+ * (2^-22 to 2^-30 of the bound of a node's sum), summed exactly. FP64, orders 2 to 5: each
+ * contribution to 1.5 * 2^-50 of the particle's own mass (first grid) or of the largest
+ * component of its m v (the others), so a node that only small weights reach can be off by
+ * more than 2^-50 of itself; order 1 and the direct BL stencil: FP64 products and sums. */
 pkmom_status pkmom_assign(pkmom_ctx *ctx, const pkmom_catalog *cat, const pkmom_params *p,
                           void *grids, void *moments_dev, void *scratch, size_t scratch_bytes,
                           void *stream);

@@ -72,9 +72,17 @@ cudaError_t launch_check_selftest(cudaStream_t s)
 }
 namespace {
 
-// Zeroed with the key table by the histogram's launch: the largest |q| of each field and the
-// moments' block counter.
-enum { kCtlQmax = 0, kCtlDone = 4, kCtlWords = 8 };
+// Zeroed with the key table by the histogram's launch: the largest |q| of each field, the
+// moments' block counter, and for FP64 2^32 less the high word of the smallest mass and of the
+// smallest largest component of a momentum (0: none, subnormals count as zero).
+enum { kCtlQmax = 0, kCtlDone = 4, kCtlLow = 5, kCtlWords = 8 };
+
+// Biased exponent of the value behind a word of kCtlLow (none: above all)
+__device__ __forceinline__ int exponent_of_least(unsigned word) { return word ? static_cast<int>((~word + 1u) >> 20) : 0x7ff; }
+// Biased exponent of an FP64 value, and whether it is zero, in integer arithmetic
+__device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
+__device__ __forceinline__ int high_word(double x) { return __double2hiint(x) & 0x7fffffff; }
 
 constexpr int kHistThreads = 256;
 constexpr int kMomentThreads = 256;
@@ -297,12 +305,14 @@ struct LaneMoments {
     T sum[NV], cmp[NV];  // the sum of a value is sum - cmp
     // FP32: max |q| of each field; FP64: the high words of the largest |q| (NaN above all)
     std::conditional_t<sizeof(T) == 4, float, int> qmax[4];
+    unsigned low[2];  // FP64: one less than the high words of kCtlLow
     __device__ __forceinline__ LaneMoments()
     {
 #pragma unroll
         for (int k = 0; k < NV; ++k) sum[k] = T(0), cmp[k] = T(0);
 #pragma unroll
         for (int f = 0; f < 4; ++f) qmax[f] = 0;
+        low[0] = low[1] = ~0u;
     }
     __device__ __forceinline__ void put(int k, T x)
     {
@@ -332,6 +342,7 @@ struct LaneMoments {
         if constexpr (MASS) {
             const T m2 = m * m, p0 = m * v0, p1 = m * v1, p2 = m * v2;
             top(0, m), top(1, p0), top(2, p1), top(3, p2);
+            if constexpr (sizeof(T) == 8) least(0, high_word(m)), least(1, p0, p1, p2);
             put(0, m);
             put(1, m2);
             put(2, p0);
@@ -348,6 +359,7 @@ struct LaneMoments {
             put(13, m2 * v1 * v2);
         } else {
             top(1, v0), top(2, v1), top(3, v2);
+            if constexpr (sizeof(T) == 8) least(1, v0, v1, v2);
             put(0, v0);
             put(1, v1);
             put(2, v2);
@@ -362,7 +374,12 @@ struct LaneMoments {
     __device__ __forceinline__ void top(int f, T x)
     {
         if constexpr (sizeof(T) == 4) qmax[f] = fmaxf(qmax[f], fabsf(x));
-        else qmax[f] = max(qmax[f], __double2hiint(x) & 0x7fffffff);
+        else qmax[f] = max(qmax[f], high_word(x));
+    }
+    __device__ __forceinline__ void least(int k, int word) { low[k] = min(low[k], static_cast<unsigned>(word) - 1u); }
+    __device__ __forceinline__ void least(int k, T a, T b, T c)
+    {
+        least(k, max(high_word(a), max(high_word(b), high_word(c))));
     }
 };
 
@@ -400,7 +417,14 @@ __device__ __forceinline__ void finish_moments(LaneMoments<T, MASS> &lm, int64_t
         if ((lane & 3) == 0) s_part[warp][8 * g + (lane >> 2)] = x;
     }
     if constexpr (!MASS && sizeof(T) == 4) lm.qmax[0] = 1.0f;
-    else if constexpr (!MASS) lm.qmax[0] = 0x3ff00000;
+    else if constexpr (!MASS) lm.qmax[0] = 0x3ff00000, lm.low[0] = 0x3ff00000 - 1;
+    if constexpr (sizeof(T) == 8) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const unsigned low = __reduce_min_sync(0xffffffffu, lm.low[k]);
+            if (lane == 0) atomicMax(qmax_bits + kCtlLow + k, ~low);
+        }
+    }
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
         // non-negative floats order like their bit patterns
@@ -851,12 +875,24 @@ k_deposit(const Record<T> *__restrict__ rec, const uint32_t *__restrict__ offset
 // FP64 grids of orders 2 to 5 are deposited in integers: offsets in the cell as 63-bit
 // fractions, weights as 62-bit ones (two words of 31 bits), values scaled by the largest
 // exponent of their field to 62 bits, and each contribution, a 62-bit integer, split into
-// words of 22, 22 and 18 bits that are summed by 32-bit shared adds. A contribution is off
-// by a few units of 2^-61 of the largest value, where an FP64 product and an FP64 sum round
-// at 2^-53 of their own; the sums are exact and do not depend on the order. The low words
-// take up to 1023 adds, then their carries are moved up. Nodes become FP64 by one rounding.
+// words of 22, 22 and 18 bits that are summed by 32-bit shared adds. The sums are exact and
+// do not depend on the order. The low words take up to 1023 adds, then their carries are
+// moved up; the high words take kIxFlush such chunks, then they are added to 64-bit sums in
+// the tile's own grid nodes. Nodes become FP64 by one rounding.
+//
+// A contribution is off by less than 6 units of 2^-61 of the scale, where FP64 products are
+// off by up to 15 roundings of 2^-53 (three weights and three products) of each value. So a
+// pass takes the particles whose mass (for the first field) and whose largest momentum
+// component (for the others) lie at most kIxGap binary orders below the scale: 6 2^-61 2^9 =
+// 2^-49.4 of themselves. What is left goes into another pass, on the scale of the largest
+// that is left, added to the nodes in FP64. With equal masses and Gaussian velocities about
+// 4 particles in 10^6 make a second pass of their tiles; masses over twelve decades take
+// five or six.
 constexpr int kIxLow = 22;         // bits of the two low words
 constexpr uint32_t kIxChunk = 1016;  // particles between carries (a multiple of 8, below 2^10)
+constexpr uint32_t kIxFlush = 7;     // 7 * 1016 contributions below 2^18 in the high word
+constexpr int kIxGap = 8;
+static_assert(kIxFlush * (kIxChunk * ((1u << 18) + 2)) < (1u << 31) - (1u << 18), "sums of the high word");
 
 // (a b) / 2^63 of 63-bit fractions (at most 2^63 itself)
 __device__ __forceinline__ unsigned long long mul63(unsigned long long a, unsigned long long b)
@@ -911,25 +947,25 @@ __device__ __forceinline__ void fixed_weights(unsigned long long t, unsigned lon
     }
 }
 
-// x 2^(62 - shift) / 2^(biased - 1022) rounded, for a finite x whose biased exponent is at
-// most `biased`: below 2^(62 - shift) in magnitude
-__device__ __forceinline__ long long fixed_value(double x, int biased, int shift)
+// x 2^62 / 2^(biased - 1022) rounded, for a finite x whose biased exponent is at most
+// `biased`: below 2^62 in magnitude
+__device__ __forceinline__ long long fixed_value(double x, int biased)
 {
     const long long bits = __double_as_longlong(x);
     const int e = static_cast<int>(bits >> 52) & 0x7ff;
     long long m = (bits & ((1ll << 52) - 1)) | (e ? 1ll << 52 : 0ll);
-    const int left = (e ? e : 1) - max(biased, 1) + 9 - shift;
+    const int left = (e ? e : 1) - max(biased, 1) + 9;
     if (left >= 0) m <<= left;
     else m = left < -62 ? 0 : (m + (1ll << (-left - 1))) >> -left;
     return bits < 0 ? -m : m;
 }
 
 // The node sum hi 2^44 + low (0 <= low < 2^44) times 2^scale as FP64, rounded once
-__device__ __forceinline__ double fixed_to_double(int hi, long long low, int scale)
+__device__ __forceinline__ double fixed_to_double(long long hi, long long low, int scale)
 {
-    // above 62 bits the lowest bits are dropped, which leaves 61
-    const int drop = max(0, 32 - __clz(hi < 0 ? ~hi : hi) - 18);
-    const long long v = (static_cast<long long>(hi) << (44 - drop)) + (low >> drop);
+    // above 62 bits the lowest bits are dropped, which leaves 61 (hi: below 2^49, n < 2^31)
+    const int drop = max(0, 64 - __clzll(hi < 0 ? ~hi : hi) - 18);
+    const long long v = (hi << (44 - drop)) + (low >> drop);
     scale += drop;
     if (v == 0) return 0.0;
     const bool neg = v < 0;
@@ -1013,11 +1049,25 @@ struct IxLanes {
     static_assert(banks_distinct() && pads_cover() && 3 * M * 2 <= WQ, "lanes in different banks, nodes in the pads");
 };
 
+// Whether a particle's mass (heavy) or momentum (fast) is part of the pass whose largest
+// exponents are base_m and base_p; what is left for later ones is noted in left.
+__device__ __forceinline__ bool in_pass(const double (&q)[4], int base_m, int base_p, int *left, bool &heavy, bool &fast)
+{
+    const int em = exponent_of(q[0]);
+    const int ep = max(exponent_of(q[1]), max(exponent_of(q[2]), exponent_of(q[3])));
+    heavy = em <= base_m && em + kIxGap >= base_m;
+    fast = ep <= base_p && ep + kIxGap >= base_p;
+    if (em + kIxGap < base_m && nonzero(q[0])) atomicMax(left, em + 1);
+    if (ep + kIxGap < base_p && (nonzero(q[1]) || nonzero(q[2]) || nonzero(q[3]))) atomicMax(left + 1, ep + 1);
+    return heavy || fast;
+}
+
 // FP64 tile-gather deposit in fixed point (see above): one particle per warp, its weights
 // evaluated by four lanes (three axes and the values) for eight particles at a time, staged in
 // shared memory and read back by all lanes. Bound by integer issue. With FP64 products and
-// shared FP64 atomics 10^6 uniform particles on 128^3 took 3.57 ms, 10^6 in halos 19.1 ms;
-// in fixed point 0.94 and 1.37 ms.
+// shared FP64 atomics 10^6 uniform particles on 128^3 took 3.58 ms, 10^6 in halos 18 to 20 ms;
+// in fixed point 0.97 and 1.46 ms, with lognormal weights (sigma 1) 1.27 and 1.89 ms, with
+// weights over twelve decades 1.72 and 2.65 ms.
 template <int M, int T0, int T1, int T2, int NT>
 __global__ void __launch_bounds__(NT)
 k_deposit_ix(const Record<double> *__restrict__ rec, const uint32_t *__restrict__ offsets,
@@ -1032,8 +1082,9 @@ k_deposit_ix(const Record<double> *__restrict__ rec, const uint32_t *__restrict_
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint32_t s_beg[C::MAXR];
     __shared__ uint32_t s_pre[C::MAXR + 1];
-    __shared__ unsigned s_rowmax;
+    __shared__ int s_left[2];  // one more than the largest exponent left (mass, momentum), 0: none
     __shared__ __align__(16) int s_stage[NW][L::NB * L::STRIDE];
+    __shared__ uint32_t s_queue[NW][L::NB + 32];
     int top[4];  // biased exponent of the largest value of each field
     bool finite = true;
 #pragma unroll
@@ -1041,8 +1092,14 @@ k_deposit_ix(const Record<double> *__restrict__ rec, const uint32_t *__restrict_
         top[f] = static_cast<int>(qmax_bits[f] >> 20);
         finite = finite && top[f] < 0x7ff;
     }
-    if (!finite || sshift != 0 || ng < C::R0 || ng < C::R1 || ng < T2 + C::HL + C::HR) {
-        // infinities and NaN, or a reach that wraps onto itself
+    // order 2 in FP64 takes no longer than four passes (10^6 particles on 128^3: 0.38 ms; one
+    // pass 0.20 ms, weights over twelve decades, six passes, 0.57 ms)
+    bool wide = false;
+    if constexpr (M == 2)
+        wide = top[0] - exponent_of_least(qmax_bits[kCtlLow]) > 3 * (kIxGap + 1) ||
+               max(top[1], max(top[2], top[3])) - exponent_of_least(qmax_bits[kCtlLow + 1]) > 3 * (kIxGap + 1);
+    if (!finite || wide || ng < C::R0 || ng < C::R1 || ng < T2 + C::HL + C::HR) {
+        // infinities and NaN, a wide range of values, or a reach that wraps onto itself
         deposit_fp64_tile<double, M, T0, T1, T2, NT, 0>(rec, offsets, ng, sshift, grids, grid_elems,
                                                         reinterpret_cast<double *>(smem_raw), s_beg, s_pre);
         return;
@@ -1054,19 +1111,12 @@ k_deposit_ix(const Record<double> *__restrict__ rec, const uint32_t *__restrict_
     const int ty = tile % nty, tx = tile / nty;
     const int t0 = tx * T0, t1 = ty * T1, t2 = tz * T2;
     int *acc = reinterpret_cast<int *>(smem_raw) + L::FRONT;  // [4 fields][low, middle, high][TNP]
-    for (int k = threadIdx.x; k < 3 * TNP; k += NT) reinterpret_cast<int4 *>(acc)[k] = make_int4(0, 0, 0, 0);
-    if (threadIdx.x == 0) s_rowmax = 0;
+    auto clear = [&]() {
+        for (int k = threadIdx.x; k < 3 * TNP; k += NT) reinterpret_cast<int4 *>(acc)[k] = make_int4(0, 0, 0, 0);
+        if (threadIdx.x < 2) s_left[threadIdx.x] = 0;
+    };
+    clear();
     const uint32_t total = build_ranges<C>(offsets, ng, sshift, t0, t1, t2, T2, s_beg, s_pre);
-    for (int r = threadIdx.x; 2 * r + 1 < C::MAXR + 1; r += NT) {
-        const uint32_t c = s_pre[2 * r + 2 <= C::MAXR ? 2 * r + 2 : C::MAXR] - s_pre[2 * r];
-        if (c) atomicMax(&s_rowmax, c);
-    }
-    __syncthreads();
-    // a node takes at most M x M rows' particles: keep the high words below 2^31
-    const float bound = kMaxWeight3<M> * 1.0001f *
-                        fminf(static_cast<float>(M * M) * static_cast<float>(s_rowmax), static_cast<float>(total));
-    int shift = 0;
-    while (bound > static_cast<float>(8000u << shift) && shift < 18) ++shift;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, a = lane & 3, sub = lane >> 2;
     const int corner = a == 0 ? t0 : a == 1 ? t1 : t2, edge = a == 0 ? T0 : a == 1 ? T1 : T2;
@@ -1078,121 +1128,203 @@ k_deposit_ix(const Record<double> *__restrict__ rec, const uint32_t *__restrict_
     const int *const sx = stage + 2 * (node ? L::dx(lane) : 0), *const sy = stage + 2 * M + 2 * (node ? L::dy(lane) : 0),
               *const sz = stage + 4 * M + 2 * (node ? L::dz(lane) : 0), *const sq = stage + L::QQ + 2 * L::field(lane);
 
-    for (uint32_t c0 = 0; c0 < total; c0 += kIxChunk) {
-        const uint32_t cnt = min(total - c0, kIxChunk);
-        if (c0) {  // carries: after at most 1023 adds
-            __syncthreads();
-            for (int k = threadIdx.x; k < 4 * TNP; k += NT) {
-                int *w = acc + (k / TNP) * 3 * TNP + k % TNP;
-                const unsigned lo = static_cast<unsigned>(w[0]);
-                const unsigned mid = static_cast<unsigned>(w[TNP]) + (lo >> kIxLow);
-                w[0] = static_cast<int>(lo & ((1u << kIxLow) - 1));
-                w[TNP] = static_cast<int>(mid & ((1u << kIxLow) - 1));
-                w[2 * TNP] += static_cast<int>(mid >> kIxLow);
-            }
-            __syncthreads();
+    // value(f, node's word in the low sums, its place in the grid) for every node of the tile
+    auto nodes = [&](auto value) {
+        for (int k = threadIdx.x; k < C::TN; k += NT) {
+            const int l2 = k % T2, l01 = k / T2;
+            const int l1 = l01 % T1, l0 = l01 / T1;
+            const int64_t gi = (static_cast<int64_t>(t0 + l0) * ng + (t1 + l1)) * (ng + 2) + t2 + l2;
+            if (!PK_IN(gi, grid_elems, kChkGrid)) continue;
+#pragma unroll
+            for (int f = 0; f < 4; ++f)
+                value(f, acc + 3 * f * TNP + l0 * L::PX + l1 * L::RW + l2, grids + f * grid_elems + gi);
         }
-        const uint32_t share = ((cnt + NW - 1) / NW + L::NB - 1) / L::NB * L::NB;
-        const uint32_t lo = min(cnt, warp * share), hi = min(cnt, lo + share);
-        int slot = lo + sub < hi ? find_slot<C::MAXR>(s_pre, c0 + lo + sub) : 0;
-        double v = 0.0, q[4] = {0.0, 0.0, 0.0, 0.0};
-        auto fetch = [&](uint32_t at) {
-            if (at + sub < hi) {
-                const uint32_t p = c0 + at + sub;
-                while (p >= s_pre[slot + 1]) ++slot;
-                const Record<double> *r = rec + s_beg[slot] + (p - s_pre[slot]);
-                v = reinterpret_cast<const double *>(r)[a];
-                if (a == 3) q[0] = r->q.x, q[1] = r->q.y, q[2] = r->q.z, q[3] = r->q.w;
-            }
+    };
+    int base_p = max(top[1], max(top[2], top[3]));
+    for (int pass = 0;; ++pass) {
+        auto emit = [&](bool high) {  // high: the grid nodes hold high sums
+            nodes([&](int f, int *w, double *g) {
+                const long long low = (static_cast<long long>(static_cast<unsigned>(w[TNP])) << kIxLow) +
+                                      static_cast<unsigned>(w[0]);
+                const long long hi = w[2 * TNP] + (low >> 44) + (high ? __double_as_longlong(*g) : 0ll);
+                const double v = fixed_to_double(hi, low & ((1ll << 44) - 1), max(top[f], 1) - 1022 - 62);
+                *g = pass ? *g + v : v;
+            });
         };
-        fetch(lo);
-        for (uint32_t at = lo; at < hi; at += L::NB) {
-            const int nb = static_cast<int>(min(hi - at, static_cast<uint32_t>(L::NB)));
-            const int packed = __shfl_sync(full, unpack_cell(v), lane | 3);
-            // the offset in the cell (in [0, 1]) as a 63-bit fraction
-            const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(a == 3 ? 0.0 : v));
-            const int e = static_cast<int>(bits >> 52) - 1012;
-            unsigned long long t = (bits & ((1ull << 52) - 1)) | 1ull << 52;
-            t = e >= 0 ? t << e : e > -53 ? t >> -e : 0ull;
-            unsigned long long w[M];
-            int first;
-            fixed_weights<M>(t, w, first);
-            int d = ((packed >> (10 * min(a, 2))) & 1023) - corner;
-            d = d < -C::HL ? d + ng : (d >= edge + C::HR ? d - ng : d);
-            d += first;
-            int word = d * pitch;
-            word += __shfl_xor_sync(full, word, 1);
-            word += __shfl_xor_sync(full, word, 2);
-            int *const st = stage + sub * L::STRIDE;
-            if (sub < nb) {
-                if (a < 3) {
-#pragma unroll
-                    for (int k = 0; k < M; ++k) {
-                        // 62 bits (one itself just below), zero outside the tile
-                        const bool in = static_cast<unsigned>(d + k) < static_cast<unsigned>(edge);
-                        const unsigned long long x = in ? min(w[k] >> 1, (1ull << 62) - 1) : 0ull;
-                        *reinterpret_cast<int2 *>(st + 2 * (a * M + k)) =
-                            make_int2(static_cast<int>(x >> 31), static_cast<int>(x & 0x7fffffffu));
-                    }
-                } else {
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) {
-                        const long long x = fixed_value(q[f], top[f], shift);
-                        *reinterpret_cast<int2 *>(st + L::QQ + 2 * f) =
-                            make_int2(static_cast<int>(x >> 31), static_cast<int>(x & 0x7fffffffll));
-                    }
-                    st[L::QQ + 8] = word;
+        const int least_m = max(top[0] - kIxGap, 0) << 20, least_p = max(base_p - kIxGap, 0) << 20;
+        bool high = false;
+        for (uint32_t c0 = 0; c0 < total; c0 += kIxChunk) {
+            const uint32_t cnt = min(total - c0, kIxChunk);
+            if (c0) {  // carries: after at most 1023 adds
+                __syncthreads();
+                for (int k = threadIdx.x; k < 4 * TNP; k += NT) {
+                    int *w = acc + (k / TNP) * 3 * TNP + k % TNP;
+                    const unsigned lo = static_cast<unsigned>(w[0]);
+                    const unsigned mid = static_cast<unsigned>(w[TNP]) + (lo >> kIxLow);
+                    w[0] = static_cast<int>(lo & ((1u << kIxLow) - 1));
+                    w[TNP] = static_cast<int>(mid & ((1u << kIxLow) - 1));
+                    w[2 * TNP] += static_cast<int>(mid >> kIxLow);
+                }
+                __syncthreads();
+                if (c0 % (kIxFlush * kIxChunk) == 0) {
+                    if (pass) emit(false);
+                    nodes([&](int, int *w, double *g) {
+                        if (pass) w[0] = w[TNP] = 0;
+                        else *g = __longlong_as_double(w[2 * TNP] + (high ? __double_as_longlong(*g) : 0ll));
+                        w[2 * TNP] = 0;
+                    });
+                    high = pass == 0;
+                    __syncthreads();
                 }
             }
-            __syncwarp();
-            fetch(at + L::NB);
-#pragma unroll 2
-            for (int p = 0; p < nb; ++p) {
-                const int o = p * L::STRIDE;
-                const int2 x = *reinterpret_cast<const int2 *>(sx + o), y = *reinterpret_cast<const int2 *>(sy + o);
-                const unsigned addr = mine + static_cast<unsigned>(4 * stage[L::QQ + 8 + o]);
-                auto mul = [](int2 u, int2 w) {  // u w / 2^62 of values in words of 31 bits
-                    const long long cross = static_cast<long long>(u.x) * w.y + static_cast<long long>(u.y) * w.x;
-                    return static_cast<long long>(u.x) * w.x + (cross >> 31);
-                };
-                auto split = [](long long u) {
-                    return make_int2(static_cast<int>(u >> 31), static_cast<int>(u & 0x7fffffffll));
-                };
-                int2 xy = split(mul(x, y));
-                if (L::USED < 32 && !node) xy = make_int2(0, 0);
-                static_for<L::NZ>([&](auto kc) {
-                    constexpr int k = decltype(kc)::value;
-                    const int2 ww = split(mul(xy, *reinterpret_cast<const int2 *>(sz + o + 2 * k)));
-                    static_for<L::NF>([&](auto fc) {
-                        constexpr int f = decltype(fc)::value;
-                        const long long c = mul(*reinterpret_cast<const int2 *>(sq + o + 2 * f), ww);
-                        if (!PK_IN(stage[L::QQ + 8 + o] + offset + L::FRONT + k + 3 * f * TNP + 2 * TNP,
-                                   L::FRONT + 12 * TNP + L::BACK, kChkShared))
-                            return;
-                        red3<4 * (k + 3 * f * TNP), 4 * TNP>(addr, static_cast<int>(c) & ((1 << kIxLow) - 1),
-                                                             static_cast<int>(c >> kIxLow) & ((1 << kIxLow) - 1),
-                                                             static_cast<int>(c >> (2 * kIxLow)));
-                    });
-                });
-            }
-            __syncwarp();
-        }
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < C::TN; k += NT) {
-        const int l2 = k % T2, l01 = k / T2;
-        const int l1 = l01 % T1, l0 = l01 / T1;
-        const int64_t gi = (static_cast<int64_t>(t0 + l0) * ng + (t1 + l1)) * (ng + 2) + t2 + l2;
-        if (!PK_IN(gi, grid_elems, kChkGrid)) continue;
+            const uint32_t share = ((cnt + NW - 1) / NW + L::NB - 1) / L::NB * L::NB;
+            const uint32_t lo = min(cnt, warp * share), hi = min(cnt, lo + share);
+            int slot = lo + sub < hi ? find_slot<C::MAXR>(s_pre, c0 + lo + sub) : 0;
+            double v = 0.0, q[4] = {0.0, 0.0, 0.0, 0.0};
+            uint32_t at = lo;
+            int waiting = 0;  // particles in the queue
+            // loads the next particles (at most eight, four lanes each) and returns their number:
+            // in the first pass the next ones, later the next of the pass (32 looked at together)
+            auto next_group = [&]() -> int {
+                if (pass == 0) {
+                    const int n = at < hi ? static_cast<int>(min(hi - at, static_cast<uint32_t>(L::NB))) : 0;
+                    if (sub < n) {
+                        const uint32_t p = c0 + at + sub;
+                        while (p >= s_pre[slot + 1]) ++slot;
+                        const Record<double> *r = rec + s_beg[slot] + (p - s_pre[slot]);
+                        v = reinterpret_cast<const double *>(r)[a];
+                        if (a == 3) q[0] = r->q.x, q[1] = r->q.y, q[2] = r->q.z, q[3] = r->q.w;
+                    }
+                    at += L::NB;
+                    return n;
+                }
+                uint32_t *const queue = s_queue[warp];
+                while (waiting < L::NB && at < hi) {
+                    bool member = false;
+                    uint32_t i = 0;
+                    if (at + lane < hi) {
+                        const int k = find_slot<C::MAXR>(s_pre, c0 + at + lane);
+                        i = s_beg[k] + (c0 + at + lane - s_pre[k]);
+                        const Vec4<double> x = rec[i].q;
+                        const double y[4] = {x.x, x.y, x.z, x.w};
+                        bool heavy, fast;
+                        member = in_pass(y, top[0], base_p, s_left, heavy, fast);
+                    }
+                    const unsigned m = __ballot_sync(full, member);
+                    if (member) queue[waiting + __popc(m & ((1u << lane) - 1u))] = i;
+                    waiting += __popc(m);
+                    at += 32;
+                    __syncwarp();
+                }
+                const int n = min(waiting, L::NB);
+                if (sub < n) {
+                    const Record<double> *r = rec + queue[sub];
+                    v = reinterpret_cast<const double *>(r)[a];
+                    if (a == 3) q[0] = r->q.x, q[1] = r->q.y, q[2] = r->q.z, q[3] = r->q.w;
+                }
+                __syncwarp();
+                waiting -= n;
+                const uint32_t moved = lane < waiting ? queue[lane + n] : 0u;
+                __syncwarp();
+                if (lane < waiting) queue[lane] = moved;
+                __syncwarp();
+                return n;
+            };
+            for (int nb = next_group(); nb;) {
+                // the particles of this pass (lane 3 of four) are staged side by side: nearly always
+                // all of them, whole, in the first pass
+                bool heavy = true, fast = true;
+                unsigned taken = 0x88888888u >> (32 - 4 * nb);
+                const bool below = high_word(q[0]) < least_m ||
+                                   max(high_word(q[1]), max(high_word(q[2]), high_word(q[3]))) < least_p;
+                if (pass || __any_sync(full, a == 3 && sub < nb && below)) {
+                    heavy = fast = false;
+                    if (a == 3 && sub < nb) in_pass(q, top[0], base_p, s_left, heavy, fast);
+                    taken = __ballot_sync(full, heavy || fast);
+                    if (!taken) {
+                        nb = next_group();
+                        continue;
+                    }
+                }
+                const int packed = __shfl_sync(full, unpack_cell(v), lane | 3);
+                // the offset in the cell (in [0, 1]) as a 63-bit fraction
+                const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(a == 3 ? 0.0 : v));
+                const int e = static_cast<int>(bits >> 52) - 1012;
+                unsigned long long t = (bits & ((1ull << 52) - 1)) | 1ull << 52;
+                t = e >= 0 ? t << e : e > -53 ? t >> -e : 0ull;
+                unsigned long long w[M];
+                int first;
+                fixed_weights<M>(t, w, first);
+                int d = ((packed >> (10 * min(a, 2))) & 1023) - corner;
+                d = d < -C::HL ? d + ng : (d >= edge + C::HR ? d - ng : d);
+                d += first;
+                int word = d * pitch;
+                word += __shfl_xor_sync(full, word, 1);
+                word += __shfl_xor_sync(full, word, 2);
+                int *const st = stage + __popc(taken & ((1u << (lane & ~3)) - 1u)) * L::STRIDE;
+                if (taken & (8u << (lane & ~3))) {
+                    if (a < 3) {
 #pragma unroll
-        for (int f = 0; f < 4; ++f) {
-            const int *w = acc + 3 * f * TNP + l0 * L::PX + l1 * L::RW + l2;
-            const long long low = (static_cast<long long>(static_cast<unsigned>(w[TNP])) << kIxLow) +
-                                  static_cast<unsigned>(w[0]);
-            grids[f * grid_elems + gi] =
-                fixed_to_double(w[2 * TNP] + static_cast<int>(low >> 44), low & ((1ll << 44) - 1),
-                                max(top[f], 1) - 1022 - 62 + shift);
+                        for (int k = 0; k < M; ++k) {
+                            // 62 bits (one itself just below), zero outside the tile
+                            const bool in = static_cast<unsigned>(d + k) < static_cast<unsigned>(edge);
+                            const unsigned long long x = in ? min(w[k] >> 1, (1ull << 62) - 1) : 0ull;
+                            *reinterpret_cast<int2 *>(st + 2 * (a * M + k)) =
+                                make_int2(static_cast<int>(x >> 31), static_cast<int>(x & 0x7fffffffu));
+                        }
+                    } else {
+#pragma unroll
+                        for (int f = 0; f < 4; ++f) {
+                            const long long x = (f ? fast : heavy) ? fixed_value(q[f], top[f]) : 0ll;
+                            *reinterpret_cast<int2 *>(st + L::QQ + 2 * f) =
+                                make_int2(static_cast<int>(x >> 31), static_cast<int>(x & 0x7fffffffll));
+                        }
+                        st[L::QQ + 8] = word;
+                    }
+                }
+                __syncwarp();
+                nb = next_group();
+#pragma unroll 2
+                for (int p = 0; p < __popc(taken); ++p) {
+                    const int o = p * L::STRIDE;
+                    const int2 x = *reinterpret_cast<const int2 *>(sx + o), y = *reinterpret_cast<const int2 *>(sy + o);
+                    const unsigned addr = mine + static_cast<unsigned>(4 * stage[L::QQ + 8 + o]);
+                    auto mul = [](int2 u, int2 w) {  // u w / 2^62 of values in words of 31 bits
+                        const long long cross = static_cast<long long>(u.x) * w.y + static_cast<long long>(u.y) * w.x;
+                        return static_cast<long long>(u.x) * w.x + (cross >> 31);
+                    };
+                    auto split = [](long long u) {
+                        return make_int2(static_cast<int>(u >> 31), static_cast<int>(u & 0x7fffffffll));
+                    };
+                    int2 xy = split(mul(x, y));
+                    if (L::USED < 32 && !node) xy = make_int2(0, 0);
+                    static_for<L::NZ>([&](auto kc) {
+                        constexpr int k = decltype(kc)::value;
+                        const int2 ww = split(mul(xy, *reinterpret_cast<const int2 *>(sz + o + 2 * k)));
+                        static_for<L::NF>([&](auto fc) {
+                            constexpr int f = decltype(fc)::value;
+                            const long long c = mul(*reinterpret_cast<const int2 *>(sq + o + 2 * f), ww);
+                            if (!PK_IN(stage[L::QQ + 8 + o] + offset + L::FRONT + k + 3 * f * TNP + 2 * TNP,
+                                       L::FRONT + 12 * TNP + L::BACK, kChkShared))
+                                return;
+                            red3<4 * (k + 3 * f * TNP), 4 * TNP>(addr, static_cast<int>(c) & ((1 << kIxLow) - 1),
+                                                                 static_cast<int>(c >> kIxLow) & ((1 << kIxLow) - 1),
+                                                                 static_cast<int>(c >> (2 * kIxLow)));
+                        });
+                    });
+                }
+                __syncwarp();
+            }
         }
+        __syncthreads();
+        const int left_m = s_left[0], left_p = s_left[1];
+        emit(high);
+        if (left_m == 0 && left_p == 0) break;
+        __syncthreads();
+        clear();
+        top[0] = left_m - 1;  // -1: no mass in the next pass
+        top[1] = top[2] = top[3] = base_p = left_p - 1;
+        __syncthreads();
     }
 }
 
