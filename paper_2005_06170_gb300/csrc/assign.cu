@@ -86,6 +86,7 @@ __device__ __forceinline__ int high_word(double x) { return __double2hiint(x) & 
 
 constexpr int kHistThreads = 256;
 constexpr int kMomentThreads = 256;
+constexpr int kLaneParticles = 512;  // particles of one FP32 sum of k_moments
 
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
@@ -301,18 +302,22 @@ k_scan_apply(uint32_t *__restrict__ counts, int64_t nkeys, const uint32_t *__res
 // m^2 v are those of m v, so only nine of the fourteen are kept.
 template <typename T, bool MASS>
 struct LaneMoments {
-    static constexpr int NV = MASS ? kMomentVals : 9;
+    static constexpr int NV = MASS ? kMomentVals : 9, NG = (NV + 7) / 8;
     T sum[NV], cmp[NV];  // the sum of a value is sum - cmp
     // FP32: max |q| of each field; FP64: the high words of the largest |q| (NaN above all)
     std::conditional_t<sizeof(T) == 4, float, int> qmax[4];
     unsigned low[2];  // FP64: one less than the high words of kCtlLow
     __device__ __forceinline__ LaneMoments()
     {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) sum[k] = T(0), cmp[k] = T(0);
+        clear();
 #pragma unroll
         for (int f = 0; f < 4; ++f) qmax[f] = 0;
         low[0] = low[1] = ~0u;
+    }
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) sum[k] = T(0), cmp[k] = T(0);
     }
     __device__ __forceinline__ void put(int k, T x)
     {
@@ -325,17 +330,40 @@ struct LaneMoments {
             sum[k] += x;
         }
     }
-    // adds another lane's sums (FP32: the pairs exactly, to 2^-48) and maxima
-    __device__ __forceinline__ void merge(const LaneMoments &o)
+    // Adds the warp's sums to total, value 8 g + k in lanes 4k .. 4k + 3 of total[g], by warp
+    // reduce-scatters (FP32: in float pairs, so that a warp does two FP64 adds instead of 70:
+    // FP64 runs at under two lanes a clock per SM on this part). Sums that leave the range of
+    // FP32 on the way across the lanes are formed again in FP64.
+    __device__ __forceinline__ void add_to(double (&total)[NG]) const
     {
 #pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            T hi = sum[k], lo = -cmp[k];
-            pair_add(hi, lo, o.sum[k], -o.cmp[k]);
-            sum[k] = hi, cmp[k] = -lo;
-        }
+        for (int g = 0; g < NG; ++g) {
+            double x;
+            if constexpr (sizeof(T) == 4) {
+                T hi[8], lo[8];
 #pragma unroll
-        for (int f = 0; f < 4; ++f) qmax[f] = max(qmax[f], o.qmax[f]);
+                for (int k = 0; k < 8; ++k) {
+                    hi[k] = 8 * g + k < NV ? sum[8 * g + k < NV ? 8 * g + k : 0] : T(0);
+                    lo[k] = 8 * g + k < NV ? -cmp[8 * g + k < NV ? 8 * g + k : 0] : T(0);
+                }
+                x = warp_scatter_sum8(hi, lo);
+                if (__any_sync(0xffffffffu, !isfinite(x))) x = scatter64(g);
+            } else {
+                x = scatter64(g);
+            }
+            total[g] += x;
+        }
+    }
+    __device__ __forceinline__ double scatter64(int g) const
+    {
+        double v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int i = 8 * g + k < NV ? 8 * g + k : 0;
+            v[k] = 8 * g + k < NV ? static_cast<double>(sum[i]) : 0.0;
+            if constexpr (sizeof(T) == 4) v[k] -= 8 * g + k < NV ? static_cast<double>(cmp[i]) : 0.0;
+        }
+        return warp_scatter_sum8(v);
     }
     __device__ __forceinline__ void add(T m, T v0, T v1, T v2)
     {
@@ -383,39 +411,23 @@ struct LaneMoments {
     }
 };
 
-// The moments of the catalogue from the lanes' sums: warp reduce-scatters (float pairs, so
-// that a warp does two FP64 adds instead of 70: FP64 runs at under two lanes a clock per SM
-// on this part), one partial per block, and the last block to finish adds the partials in a
-// fixed order into out (pkmom_moments). done: a zeroed counter. As FP64 butterflies in 1216
-// blocks and a separate kernel the same sums took 80 us whatever the catalogue's size.
+// The moments of the catalogue from the warps' sums (total: LaneMoments::add_to) and the lanes'
+// maxima: one partial per block, and the last block to finish adds the partials in a fixed
+// order into out (pkmom_moments). done: a zeroed counter. As FP64 butterflies in 1216 blocks
+// and a separate kernel the same sums took 80 us whatever the catalogue's size.
 template <typename T, bool MASS>
-__device__ __forceinline__ void finish_moments(LaneMoments<T, MASS> &lm, int64_t n, double *__restrict__ partials,
-                                               unsigned *__restrict__ qmax_bits, unsigned *__restrict__ done,
-                                               double *__restrict__ out)
+__device__ __forceinline__ void finish_moments(LaneMoments<T, MASS> &lm,
+                                               const double (&total)[LaneMoments<T, MASS>::NG], int64_t n,
+                                               double *__restrict__ partials, unsigned *__restrict__ qmax_bits,
+                                               unsigned *__restrict__ done, double *__restrict__ out)
 {
-    constexpr int NV = LaneMoments<T, MASS>::NV, NG = (NV + 7) / 8;
+    constexpr int NV = LaneMoments<T, MASS>::NV, NG = LaneMoments<T, MASS>::NG;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     __shared__ double s_part[kMomentThreads / 32][8 * NG];
     __shared__ bool s_last;
 #pragma unroll
-    for (int g = 0; g < NG; ++g) {
-        double x;
-        if constexpr (sizeof(T) == 4) {
-            T hi[8], lo[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                hi[k] = 8 * g + k < NV ? lm.sum[8 * g + k < NV ? 8 * g + k : 0] : T(0);
-                lo[k] = 8 * g + k < NV ? -lm.cmp[8 * g + k < NV ? 8 * g + k : 0] : T(0);
-            }
-            x = warp_scatter_sum8(hi, lo);
-        } else {
-            double v[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = 8 * g + k < NV ? lm.sum[8 * g + k < NV ? 8 * g + k : 0] : T(0);
-            x = warp_scatter_sum8(v);
-        }
-        if ((lane & 3) == 0) s_part[warp][8 * g + (lane >> 2)] = x;
-    }
+    for (int g = 0; g < NG; ++g)
+        if ((lane & 3) == 0) s_part[warp][8 * g + (lane >> 2)] = total[g];
     if constexpr (!MASS && sizeof(T) == 4) lm.qmax[0] = 1.0f;
     else if constexpr (!MASS) lm.qmax[0] = 0x3ff00000, lm.low[0] = 0x3ff00000 - 1;
     if constexpr (sizeof(T) == 8) {
@@ -474,8 +486,18 @@ k_moments(const T *__restrict__ vx, const T *__restrict__ vy, const T *__restric
           unsigned *__restrict__ done, double *__restrict__ out)
 {
     LaneMoments<T, MASS> lm;
+    double total[LaneMoments<T, MASS>::NG] = {};
     const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i0 < n; i0 += 4 * step) {
+    int count = 0;
+    // (the warp's lanes run the same iterations)
+    for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i0 - (threadIdx.x & 31) < n;
+         i0 += 4 * step) {
+        if (sizeof(T) == 4 && count == kLaneParticles / 4) {  // FP32 sums of at most kLaneParticles
+            lm.add_to(total);
+            lm.clear();
+            count = 0;
+        }
+        ++count;
         T m[4], a[4], b[4], c[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -491,14 +513,15 @@ k_moments(const T *__restrict__ vx, const T *__restrict__ vy, const T *__restric
 #pragma unroll
         for (int k = 0; k < 4; ++k) lm.add(m[k], a[k], b[k], c[k]);
     }
-    finish_moments<T, MASS>(lm, n, partials, qmax_bits, done, out);
+    lm.add_to(total);
+    finish_moments<T, MASS>(lm, total, n, partials, qmax_bits, done, out);
 }
 
 // FP32 interleaved (n, 3) velocities, 16-byte aligned: four particles per thread read
 // as three 128-bit loads ((v0x v0y v0z v1x) (v1y v1z v2x v2y) (v2z v3x v3y v3z)), and
 // four masses as one. The particles are dealt to `lanes` sums, lane v taking the quads v,
 // v + lanes, ..., and lane v < 32 the v-th of the n % 4 last particles, whatever the number
-// of threads (a thread takes several lanes and merges their pairs): a compensated sum of
+// of threads (a thread takes several lanes, one after another): a compensated sum of
 // values that cancel, such as the momentum of a catalogue without bulk flow, depends on how
 // they are dealt, and the size of the launch should not matter.
 template <bool MASS>
@@ -512,10 +535,12 @@ k_moments_v3(const float *__restrict__ v, const float *__restrict__ mass, int64_
     const float4 *v4 = reinterpret_cast<const float4 *>(v);
     const float4 *m4 = reinterpret_cast<const float4 *>(mass);
     const int64_t used = nq > 32 ? (nq < lanes ? nq : lanes) : 32;  // the other lanes are empty
-    LaneMoments<float, MASS> all;
-    for (int64_t vl = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; vl < used; vl += step) {
-        LaneMoments<float, MASS> lm;
-        for (int64_t q = vl; q < nq; q += lanes) {
+    LaneMoments<float, MASS> lm;
+    double total[LaneMoments<float, MASS>::NG] = {};
+    for (int64_t vl = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; vl - (threadIdx.x & 31) < used;
+         vl += step) {  // (the warp's lanes run the same iterations; `used` is no multiple of 32)
+        lm.clear();
+        for (int64_t q = vl < used ? vl : nq; q < nq; q += lanes) {
             const float4 a = v4[3 * q], b = v4[3 * q + 1], c = v4[3 * q + 2];
             float4 mm = make_float4(1.f, 1.f, 1.f, 1.f);
             if constexpr (MASS) mm = m4[q];
@@ -530,9 +555,9 @@ k_moments_v3(const float *__restrict__ v, const float *__restrict__ mass, int64_
             if constexpr (MASS) m = mass[i];
             lm.add(m, v[3 * i], v[3 * i + 1], v[3 * i + 2]);
         }
-        all.merge(lm);
+        lm.add_to(total);
     }
-    finish_moments<float, MASS>(all, n, partials, qmax_bits, done, out);
+    finish_moments<float, MASS>(lm, total, n, partials, qmax_bits, done, out);
 }
 
 // ------------------------------------------------------------------ scatter
