@@ -1409,10 +1409,28 @@ __device__ __forceinline__ uint32_t cell_chunk(const Record<float> *__restrict__
         }
     };
     uint32_t i = i0;
-    if (z >= 0) {
-        for (int n = 0; i < i1 && n < kCellFlush; ++i) {
-            const Record<float> r = load_record(rec + i);
-            if ((unpack_cell(r.u.w) >> 20) == z) add(r), ++n;  // warp-uniform
+    if (z >= 0) {  // the cells of 32 records are read together, then the records of this cell
+        const uint32_t lane = threadIdx.x & 31;
+        auto cell_z = [&](uint32_t at) { return at + lane < i1 ? unpack_cell(rec[at + lane].u.w) >> 20 : -1; };
+        int next = cell_z(i);
+        for (int n = 0; i < i1; i += 32) {
+            unsigned m = __ballot_sync(0xffffffffu, next == z);
+            n += __popc(m);
+            if (n > kCellFlush) break;  // the next chunk starts with these
+            next = cell_z(i + 32);
+            auto take = [&]() {
+                const uint32_t k = i + __ffs(static_cast<int>(m)) - 1;
+                m &= m - 1u;
+                return load_record(rec + k);
+            };
+            while (__popc(m) >= 4) {  // four loads in flight
+                const Record<float> r0 = take(), r1 = take(), r2 = take(), r3 = take();
+                add(r0);
+                add(r1);
+                add(r2);
+                add(r3);
+            }
+            while (m) add(take());
         }
         i1 = i;
     }
@@ -1483,7 +1501,7 @@ __device__ __forceinline__ void deposit_cells_path(const Record<float> *__restri
         const int oa = lxa * px + ly * rw + lz, ob = (lxa + 2) * px + ly * rw + lz;
         for (uint32_t i0 = beg; i0 < end;) {
             int a[4], b[4];
-            i0 = sshift ? cell_chunk(rec, i0, end, pc, fine, shift, a, b, z)
+            i0 = T2 >= 16 && sshift ? cell_chunk(rec, i0, end, pc, fine, shift, a, b, z)
                         : cell_chunk(rec, i0, min(end, i0 + kCellFlush), pc, fine, shift, a, b);
 #pragma unroll
             for (int f = 0; f < 4; ++f) {
@@ -1985,12 +2003,16 @@ __device__ __forceinline__ void fx_tile(const Record<float> *__restrict__ rec, c
         __syncthreads();
         if (threadIdx.x == 0) s_rowmax = s_reached = s_inner = s_unsure = 0;
         __syncthreads();
-        for (int r = threadIdx.x; r < C::R0 * C::R1; r += NT) {
+        auto row_of = [&](int r) {  // offsets of the runs of a row
             int a0 = t0 - C::HL + r / C::R1, a1 = t1 - C::HL + r % C::R1;
             a0 = a0 < 0 ? a0 + ng : (a0 >= ng ? a0 - ng : a0);
             a1 = a1 < 0 ? a1 + ng : (a1 >= ng ? a1 - ng : a1);
-            const uint32_t *row = offsets + ((static_cast<int64_t>(a0) * ng + a1) * ng >> sshift);
-            const uint32_t c = row[(t2 + T2) >> sshift] - row[t2 >> sshift];
+            return offsets + ((static_cast<int64_t>(a0) * ng + a1) * ng >> sshift);
+        };
+        const int in0 = t2 >> sshift, in1 = (t2 + T2) >> sshift;  // the runs inside the tile
+        for (int r = threadIdx.x; r < C::R0 * C::R1; r += NT) {
+            const uint32_t *row = row_of(r);
+            const uint32_t c = row[in1] - row[in0];
             if (c) atomicAdd(&s_reached, c), atomicMax(&s_inner, c);
         }
         __syncthreads();
@@ -2011,9 +2033,8 @@ __device__ __forceinline__ void fx_tile(const Record<float> *__restrict__ rec, c
             d = d < -C::HL ? d + ng : (d >= T2 + C::HR ? d - ng : d);
             return d >= -C::HL && d < T2 + C::HR ? 1u : 0u;
         };
-        for (int s0 = 0; s0 < C::MAXR && unsure; s0 += NT) {
-            const int slot = s0 + static_cast<int>(threadIdx.x);
-            const uint32_t b = slot < C::MAXR ? s_beg[slot] : 0u, len = slot < C::MAXR ? s_pre[slot + 1] - s_pre[slot] : 0u;
+        // particles of a range within reach: short ranges by their thread, long ones by the warp
+        auto reaching = [&](uint32_t b, uint32_t len) {
             uint32_t c = 0;
             if (len <= 8u)
                 for (uint32_t i = 0; i < len; ++i) c += within(b + i);
@@ -2025,8 +2046,19 @@ __device__ __forceinline__ void fx_tile(const Record<float> *__restrict__ rec, c
                 n = __reduce_add_sync(0xffffffffu, n);
                 if (lane == l) c = n;
             }
-            const uint32_t row = c + __shfl_xor_sync(0xffffffffu, c, 1);  // a row's two pieces
-            if (c) atomicAdd(&s_reached, c), atomicMax(&s_rowmax, row);
+            return c;
+        };
+        // only the runs on either side of the tile hold particles out of reach
+        const int below = (C::HL + (1 << sshift) - 1) >> sshift, above = (C::HR + (1 << sshift) - 1) >> sshift;
+        const int lo0 = (in0 ? in0 : ng >> sshift) - below, up0 = t2 + T2 == ng ? 0 : in1;
+        for (int r0 = 0; r0 < C::R0 * C::R1 && unsure; r0 += NT) {
+            const int r = r0 + static_cast<int>(threadIdx.x);
+            const bool any = r < C::R0 * C::R1;
+            const uint32_t *row = any ? row_of(r) : offsets;
+            uint32_t c = any ? row[in1] - row[in0] : 0u;
+            c += reaching(row[lo0], any ? row[lo0 + below] - row[lo0] : 0u);
+            c += reaching(row[up0], any ? row[up0 + above] - row[up0] : 0u);
+            if (c) atomicAdd(&s_reached, c), atomicMax(&s_rowmax, c);
         }
         __syncthreads();
         reached = s_reached;
@@ -2155,7 +2187,7 @@ __device__ __forceinline__ void fx_tile(const Record<float> *__restrict__ rec, c
 #pragma unroll
             for (int k = 0; k < KP; ++k) {
                 const int g = key[k] & 31, r = key[k] >> 5;
-                const uint32_t from = __shfl_sync(0xffffffffu, last, g);
+                const uint32_t from = maxc > kRanks ? __shfl_sync(0xffffffffu, last, g) : 0u;
                 if (key[k] < 0) continue;
                 s_idx[r < kListRankMax ? s_rbase[r] + __popc(s_rmask[r] & ((1u << g) - 1u)) : from + r - kListRankMax] =
                     idx[k];
