@@ -1353,7 +1353,7 @@ k_deposit_ix(const Record<double> *__restrict__ rec, const uint32_t *__restrict_
     }
 }
 
-// Cell-block path of the FP32 deposit for dense tiles (cubic order, per-cell keys): one
+// Cell-block path of the FP32 deposit for dense tiles (cubic order): one
 // warp per occupied cell of the reach; lane l owns stencil nodes (dx, dy, dz) with
 // dz = l & 3, dy = (l >> 2) & 3, dx = (l >> 4) and (l >> 4) + 2, evaluates its weight
 // pieces by Horner's rule with lane-constant coefficients, sums up to kCellFlush of the
@@ -1724,7 +1724,10 @@ struct CoopLanes {
     static constexpr int QW = 3 * WP;                  // the scaled values, then the node word
     static constexpr int STRIDE = M == 4 ? 20 : 32;    // staged words per particle
     static constexpr int NB = 8;                       // particles staged at a time
-    static constexpr int COST = M == 4 ? 16 : 30;      // about the wavefronts of a particle
+    // About the wavefronts of a particle. Whole calls with half and twice of it over this: 10 M
+    // uniform particles on 200^3 1.05 and 1.01 (order 4), 1.41 and 1.00 (order 5); 1 M in halos on
+    // 128^3 1.03 and 1.21, 1.06 and 1.03
+    static constexpr int COST = M == 4 ? 16 : 30;
     __host__ __device__ static constexpr int dx(int lane) { return M == 4 ? (lane >> 2) & 3 : lane / 5; }
     __host__ __device__ static constexpr int dy(int lane) { return M == 4 ? lane & 3 : lane % 5; }
     __host__ __device__ static constexpr int half(int lane) { return M == 4 ? lane >> 4 : 0; }
@@ -1891,25 +1894,29 @@ __device__ __forceinline__ void coop_deposit(const Record<float> *__restrict__ r
 // Tile-gather deposit for FP32 grids with 32-bit integer (fixed-point) shared-memory
 // atomics (about three times the throughput of FP32 shared atomics on this part).
 //
-// Work split: tiles whose reach holds few particles (sparse catalogues) list them in
-// shared memory, reordered so that 32 consecutive entries have their first stencil nodes
-// in different banks, and warps take consecutive chunks of 32 (banked_particle: every
-// node at an immediate offset, nodes outside the tile adding exactly 0). Other
-// tiles: each warp walks its own contiguous chunk of the tile's particle list 32 at a
-// time, lane j taking the j-th particle of each step, node by node; tiles with more than
-// two particles per reach cell (cubic order) take the cell-block path. The accumulator
-// layout is FxLayout.
+// Work split: orders 4 and 5, and sparse catalogues at orders 1 to 3, list a tile's
+// particles in shared memory, a few thousand at a time, and deposit them a particle per lane
+// (banked_particle: the list reordered so that 32 consecutive entries have their first
+// stencil nodes in different banks, every node at an immediate offset, nodes outside the
+// tile adding exactly 0) or, crowded lists at orders 4 and 5, a particle per warp
+// (coop_deposit). The rest (orders 1 to 3 from half a particle per cell on or with a list too
+// long, the direct BL stencil, a reach that wraps onto itself) goes node by node: each warp
+// walks its own contiguous chunk of the tile's particles, lane j taking the j-th of each 32.
+// Tiles with more than two particles per reach cell (cubic order) take the cell-block path.
+// The accumulator layout is FxLayout.
 //
 // Fixed point: field f of the tile uses the scale 2^s_f with
 //   B_f 2^s_f < 2^30,   B_f = w3 * min(M^2 * largest row count, particle count) * max |q_f|
 // over the tile's reach (w3 = the largest product of three weights; a node receives from
 // at most M^2 cell rows, each contributing at most `largest row count` particles, and
-// from no more than all of them; max |q_f| over the catalogue), so no node sum can overflow, and also max |q_f| w3 2^s_f < 2^22, so that
-// every contribution is rounded to an integer by one FFMA against 1.5 * 2^23 (round to
+// from no more than all of them; max |q_f| over the catalogue), so no node sum can
+// overflow, and also max |q_f| w3 2^s_f < 2^22, so that every contribution is rounded to an integer by one FFMA against 1.5 * 2^23 (round to
 // nearest even, one rounding of the exact product). The bound depends only on counts
 // and maxima, and integer sums do not depend on order: the grids are the same whatever
 // order the sort leaves particles of one cell in.
-constexpr int kListRankMax = 128;  // ranks within a bank group that the list is ordered by
+// Ranks within a bank group that the list is ordered by (64: 5 M uniform particles on 256^3 at
+// order 4 1.06 times as long, others the same).
+constexpr int kListRankMax = 128;
 
 // One tile of the FP32 gather deposit (the body of k_deposit_fx, and of each work item
 // of its persistent batched form k_deposit_fx_batch). The whole CTA takes part; its
@@ -2545,11 +2552,11 @@ __device__ __forceinline__ void home_pair(unsigned acc_s, const Record<float> (&
     for (int j = 0; j < CP; ++j) qp[j][0] = f2_pack(q[j][0], q[j][1]), qp[j][1] = f2_pack(q[j][2], q[j][3]);
     const f32x2 mg = f2_pack(kMagic, kMagic);
     // buffer index of node (cx - 1 + dx, cy - 1 + dy, CP m - 1 + i) is (cx + dx) PX + (cy + dy) PY + CP m + i.
-    // The dx loop is rolled (a short body for the instruction cache): the weights of the
-    // current dx are kept in slot 0 by rotating them.
-    // the lane's last node (3, 3 node columns on) must lie in the buffer
+    // The lane's last node (3, 3 node columns on) must lie in the buffer.
     if (!PK_IN((cx + 3) * kHomePX + (cy + 3) * kHomePY + CP * m + CP + 2, kHomeField, kChkShared)) return;
     unsigned base = acc_s + 4u * static_cast<unsigned>(cx * kHomePX + cy * kHomePY + CP * m);
+    // rolled (a short body for the instruction cache): the weights of the current dx are kept in
+    // slot 0 by rotating them
 #pragma unroll 1
     for (int dx = 0; dx < 4; ++dx) {
         static_for<4>([&](auto dyc) {
@@ -2825,14 +2832,8 @@ k_deposit_home(const Record<float> *__restrict__ rec, const uint32_t *__restrict
             }
             const int cx = 2 * (blk / BY) + xl, cy = kHomeColY * (blk % BY) + yl;
             const int64_t key = (static_cast<int64_t>(t0 + cx) * ng + (t1 + cy)) * ng + (t2 + CP * m);
-            o[0] = offsets[key];
-            if constexpr (CP == 4) {
-                const uint4 v = *reinterpret_cast<const uint4 *>(offsets + key + 1);
-                o[1] = v.x, o[2] = v.y, o[CP - 1] = v.z, o[CP] = v.w;
-            } else {
-                const uint2 v = *reinterpret_cast<const uint2 *>(offsets + key + 1);
-                o[1] = v.x, o[2] = v.y;
-            }
+            const uint2 v = *reinterpret_cast<const uint2 *>(offsets + key + 1);
+            o[0] = offsets[key], o[1] = v.x, o[2] = v.y;
         };
         uint32_t on[CP + 1];
         cell_offsets(warp, on);  // loads run one block ahead

@@ -185,9 +185,16 @@ AssignPlan plan_assign(const pkmom_params &p, int64_t n, int num_sms, int tile_o
     // stick out of its reach. Not beyond the density where the row bound of a tile (order^2
     // times its fullest row's particles) usually passes 256, above which a tile has to look
     // closer (fx_tile). 512^3 particles on 1024^3, histogram + scan + scatter + deposit: one
-    // cell a key 24.96 ms, two 23.01, four 22.42; 0.83 M on 384^3: 0.88, 0.81, 0.76.
+    // cell a key 24.96 ms, two 23.01, four 22.42; 0.83 M on 384^3: 0.88, 0.81, 0.76. Whole calls
+    // with one cell a key over several, uniform particles: 1.03 to 1.14 at orders 1 to 3 from
+    // 160^3 on, 1.03 to 1.05 at orders 4 and 5; one clump of nine tenths of the particles: 1.2 to
+    // 2.2 at orders 2 and 3, 0.76 to 1.09 at order 1 (below 1 where it lies on a tile's corner).
+    // At order 4 a dense tile looks at a run once per cell of it: halos 0.94 to 0.96 and a clump
+    // 0.81 to 0.90 on 128^3, against 1.01 to 1.02 for uniform particles; 1.02 and 0.96, 0.93 to
+    // 1.17, 1.03 to 1.05 on 192^3. So cubic order takes several cells from 192^3 on.
     int sshift = 0;
-    if (p.precision == PKMOM_F32 && p.bl_radius == 0 && pl.tile != kHomeTile && td[2] >= 16) {
+    if (p.precision == PKMOM_F32 && p.bl_radius == 0 && pl.tile != kHomeTile && td[2] >= 16 &&
+        (p.order != 4 || p.ng >= 192)) {
         for (int k = 2; k > 0 && sshift == 0; --k) {
             const double mean = ppc * (td[2] + 4.0 + (1 << k));  // particles of a row of the runs
             if (p.order * p.order * (mean + 4.5 * std::sqrt(mean) + 2.0) <= 256.0) sshift = k;
@@ -197,7 +204,9 @@ AssignPlan plan_assign(const pkmom_params &p, int64_t n, int num_sms, int tile_o
     // FP32 gather tiles list their particles in shared memory: room for about twice the
     // expected count of a tile's reach, at most 2048 (longer ones go 2048 at a time).
     // Orders 1 to 3 list sparse catalogues only: from half a particle per cell on, adding
-    // node by node was faster (TSC, 5 M particles on 200^3: 0.40 against 0.42 ms)
+    // node by node was faster or the same (deposit of 5 M particles on 200^3 at order 3: 0.40
+    // against 0.42 ms; whole calls, listed over node by node: 10 M on 200^3 1.03, 0.97 and 1.00 at
+    // orders 1 to 3, 1 M in halos on 128^3 0.98, 1.02 and 1.04)
     const double reach = double(td[0] + 3) * (td[1] + 3) * (td[2] + 3);
     if (p.precision == PKMOM_F32 && (ppc < 0.5 || p.order >= 4)) {
         const double want = 2.0 * ppc * reach + 64.0;

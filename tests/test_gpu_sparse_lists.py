@@ -48,15 +48,16 @@ def _grids(pk, pos, vel, L, ng, order, tuning, checked):
 
 # 48^3, 16^3 tiles, lists of 256: 130 to 200 particles in a cell of two tiles, strays in the
 # cells of their runs of four beyond the reach (12 to 15 below the corner at 16, 32 to 35 above;
-# 44 to 47 and 16 to 19 around the box's corner). 64^3, 16 x 16 x 32 tiles, lists of 4096: bank
+# 4 to 1 below and 16 to 19 above the box's corner); cubic order has such keys from 192^3 on. 64^3, 16 x 16 x 32 tiles, lists of 4096: bank
 # groups beyond 128 without a crowded cell.
 @pytest.mark.parametrize("order,ng,tuning,kind", [(o, 48, (-1, -1), k) for o in (1, 2, 3, 4, 5) for k in (130, 200)] +
-                         [(o, 64, (1, 4096), 0) for o in (1, 2, 3, 4, 5)])
+                         [(4, 192, (-1, -1), 200)] + [(o, 64, (1, 4096), 0) for o in (1, 2, 3, 4, 5)] +
+                         [(4, 192, (1, 4096), 0)])
 def test_particles_out_of_reach_stay_out(gpu_lib, order, ng, tuning, kind):
     L = 96.0
     if kind:
         cells = _crowd((20, 21, 20), kind, (12, 13, 14, 15, 32, 33, 34, 35))
-        cells += _crowd((3, 2, 1), kind, (44, 45, 46, 47, 16, 17, 18, 19))
+        cells += _crowd((3, 2, 1), kind, (ng - 4, ng - 3, ng - 2, ng - 1, 16, 17, 18, 19))
     else:
         rng = np.random.Generator(np.random.PCG64(2))
         cells = np.concatenate([rng.integers((18, 18, 34), (30, 30, 62), (3850, 3)),
@@ -71,3 +72,22 @@ def test_particles_out_of_reach_stay_out(gpu_lib, order, ng, tuning, kind):
     for f in range(4):
         tol = 3.0 * np.sqrt(n) * 2.0 * W3[order] * n * q[f] / 2.0 ** 30 + 1e-6 * (np.abs(ref[f]).max() + q[f])
         assert np.max(np.abs(listed[0][f] - ref[f])) <= tol, f
+
+
+@pytest.mark.parametrize("at", [0.0, 7.5])
+def test_dense_tiles_of_runs(gpu_lib, at):
+    """Cubic order, keys of four cells, a clump on a tile's corner (the box's) and inside a tile:
+    dense tiles find a cell's particles, some with more than 256, in its run. A lost or misplaced
+    particle changes a node by 0.01 to 1 of its value."""
+    L, ng, n = 192.0, 192, 60000
+    rng = np.random.Generator(np.random.PCG64(8))
+    pos = np.mod(rng.normal(at, 1.4, (n, 3)), L).astype(np.float32)
+    pos[pos >= np.float32(L)] = 0
+    vel = rng.normal(0.0, 100.0, (n, 3)).astype(np.float32)
+    got = [_grids(gpu_lib, pos, vel, L, ng, 4, (-1, -1), checked) for checked in (False, True)]
+    ref = est.assign(pos, vel, None, L=L, ng=ng, order=4)
+    q = [1.0] + [np.abs(vel[:, a]).max() for a in range(3)]
+    for f in range(4):
+        tol = 3.0 * np.sqrt(n) * 2.0 * W3[4] * n * q[f] / 2.0 ** 30 + 1e-6 * (np.abs(ref[f]).max() + q[f])
+        for g in got:
+            assert np.max(np.abs(g[f] - ref[f])) <= tol, f
