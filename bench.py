@@ -59,7 +59,7 @@ DEFAULT = "zeldovich512_ng512"
 # capture of the current kernels; a stage whose kernels change drops its entry until
 # it is captured again
 MEASURED_TRAFFIC = {
-    ("zeldovich512_ng512", "deposit"): (8 * (630.6 + 416.6 + 457.8 + 168.7) * 1e6,
+    ("zeldovich512_ng512", "deposit"): (8 * (630.8 + 416.5 + 457.6 + 168.8) * 1e6,
                                         "ncu dram__bytes_read.sum + dram__bytes_write.sum of k_deposit_home and "
                                         "k_home_fixup, one launch of each at 256^3 particles on 256^3 "
                                         "(profiles/own_kernels.md), times 8"),
@@ -75,7 +75,7 @@ MEASURED_TRAFFIC = {
 # the current kernel on the 256^3 workload, scaled to other workloads by particle count
 # (the same work per particle at one particle per cell)
 MEASURED_INSTRUCTIONS = {
-    "k_deposit_home": (544.75e6, 256 ** 3, "ncu smsp__inst_executed.sum of k_deposit_home, 256^3 Zel'dovich "
+    "k_deposit_home": (544.7e6, 256 ** 3, "ncu smsp__inst_executed.sum of k_deposit_home, 256^3 Zel'dovich "
                                          "particles on 256^3 (profiles/own_kernels.md), scaled by particles"),
 }
 # configs 4 and 5 run through their own drivers below

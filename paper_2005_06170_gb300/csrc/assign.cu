@@ -2104,8 +2104,33 @@ __device__ __forceinline__ void fx_tile(const Record<float> *__restrict__ rec, c
     const uint32_t chunk = min(static_cast<uint32_t>(list_cap), static_cast<uint32_t>(KP * NT));
     const bool use_list = M >= 4 || (sparse && total <= chunk);
     const bool long_rows = s_rowmax > 24u;
-    if (BLR == 0 && list_cap > 0 && use_list && !dense && ng >= C::R0 && ng >= C::R1 &&
-        ng >= T2 + C::HL + C::HR) {
+    const bool unwrapped = ng >= C::R0 && ng >= C::R1 && ng >= T2 + C::HL + C::HR;
+    if constexpr (COOP && M == 5 && T0 == 8) {
+        // Order 5 on tiles of 8 x 8 rows, crowded (one row holds five times the mean of the
+        // rows, or a list is no longer than the particles of 64 cells): a particle per warp
+        // straight from the ranges. Listing them first takes as long again here, since a
+        // particle is listed by four tiles and a tile's last list is often the whole kernel's
+        // tail: whole calls over those with a branch per node and no list, 10^5 particles in
+        // halos on 56^3 1.15 listed, 0.77 so; 3.4 10^5 on 72^3 1.16 and 0.81; 4.3 10^6 on 168^3
+        // 0.93 and 0.87; a clump of 1.1 10^6 on 200^3 1.5 and 0.92. With eight times the mean
+        // 10^5 on 88^3 take 1.10 (0.76 with five). Cubic order and 16^3 tiles, whose halo
+        // particles are fewer, are faster listed (2.5 10^6 in halos on 256^3 0.72 against 0.79).
+        const bool crowded = s_rowmax * static_cast<uint32_t>(C::R0 * C::R1) > 5u * total || total / NREACH > chunk / 64u;
+        if (list_cap > 0 && total > 256u && crowded && unwrapped) {
+            const uint32_t share = ((total + NW - 1) / NW + 7u) & ~7u, lo = min(total, warp * share);
+            const uint32_t n = min(share, total - lo);
+            int slot = static_cast<uint32_t>(lane >> 2) < n ? find_slot<C::MAXR>(s_pre, lo + (lane >> 2)) : 0;
+            coop_deposit<M, T0, T1, T2, C::HL, C::HR>(
+                rec,
+                [&](uint32_t p) {
+                    while (lo + p >= s_pre[slot + 1]) ++slot;
+                    return s_beg[slot] + (lo + p - s_pre[slot]);
+                },
+                n, ng, t0, t1, t2, acc, s_stage[warp], sc0, sc1, sc2, sc3);
+            done = true;
+        }
+    }
+    if (BLR == 0 && list_cap > 0 && use_list && !dense && !done && unwrapped) {
         for (uint32_t c0 = 0; c0 < total; c0 += chunk) {
             const uint32_t cnt = min(chunk, total - c0);
             if (c0) {

@@ -36,7 +36,8 @@ def _far(pos, L, ng, bad):
 # 48^3: 16^3 tiles, keys of four cells; 40^3: 8^3 tiles, sparse and at two particles a cell
 # (lists in several parts); "crowd": half of the particles in a cell (one particle a warp)
 @pytest.mark.parametrize("order", [1, 2, 3, 4, 5])
-@pytest.mark.parametrize("ng,n,kind", [(48, 3000, ""), (40, 3000, ""), (40, 128000, ""), (48, 1200, "crowd")])
+@pytest.mark.parametrize("ng,n,kind", [(48, 3000, ""), (40, 3000, ""), (40, 128000, ""), (48, 1200, "crowd"),
+                                       (40, 1200, "crowd")])
 @pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
 def test_nonfinite_velocities_stay_in_place(gpu_lib, order, ng, n, kind, value):
     L = 100.0

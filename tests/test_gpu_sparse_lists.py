@@ -91,3 +91,29 @@ def test_dense_tiles_of_runs(gpu_lib, at):
         tol = 3.0 * np.sqrt(n) * 2.0 * W3[4] * n * q[f] / 2.0 ** 30 + 1e-6 * (np.abs(ref[f]).max() + q[f])
         for g in got:
             assert np.max(np.abs(g[f] - ref[f])) <= tol, f
+
+
+@pytest.mark.parametrize("kind", ["row", "clump", "edge"])
+def test_crowded_small_tiles_at_order_five(gpu_lib, kind):
+    """8^3 tiles at order 5: crowded tiles are deposited a particle per warp straight from their
+    ranges (one row far above the others; many particles a cell; a clump on the box's corner,
+    whose ranges wrap), the others from lists."""
+    L, ng, n = 80.0, 40, 6000
+    rng = np.random.Generator(np.random.PCG64(5))
+    cells = rng.integers(0, ng, (n, 3))
+    m = n // 2
+    if kind == "row":
+        cells[:m, :2] = 21, 13
+    if kind == "clump":
+        cells[:] = rng.integers(16, 19, (n, 3))
+    if kind == "edge":
+        cells[:m] = rng.integers(-2, 2, (m, 3)) % ng
+    pos, vel = _cells(cells, L, ng, seed=7)
+    got = [_grids(gpu_lib, pos, vel, L, ng, 5, (-1, -1), checked) for checked in (False, True)]
+    by_node = _grids(gpu_lib, pos, vel, L, ng, 5, (-1, 0), False)
+    assert np.array_equal(got[0], by_node) and np.array_equal(got[1], by_node)
+    ref = est.assign(pos, vel, None, L=L, ng=ng, order=5)
+    q = [1.0] + [np.abs(vel[:, a]).max() for a in range(3)]
+    for f in range(4):
+        tol = 3.0 * np.sqrt(n) * 2.0 * W3[5] * n * q[f] / 2.0 ** 30 + 1e-6 * (np.abs(ref[f]).max() + q[f])
+        assert np.max(np.abs(got[0][f] - ref[f])) <= tol, f
