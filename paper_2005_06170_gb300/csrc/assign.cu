@@ -1726,8 +1726,10 @@ struct CoopLanes {
     static constexpr int NB = 8;                       // particles staged at a time
     // About the wavefronts of a particle. Whole calls with half and twice of it over this: 10 M
     // uniform particles on 200^3 1.05 and 1.01 (order 4), 1.41 and 1.00 (order 5); 1 M in halos on
-    // 128^3 1.03 and 1.21, 1.06 and 1.03
-    static constexpr int COST = M == 4 ? 16 : 30;
+    // 128^3 1.03 and 1.21, 1.06 and 1.03. On 8^3 tiles, where a particle's visits are mostly zero
+    // adds, order 4 with 16, 20 and 26 over a branch per node: lattices of 0.2 a cell on 264^3 1.014,
+    // 1.002 and 0.997, uniform ones 0.978, 0.970 and 0.966, in halos 0.77, 0.79 and 0.81
+    static constexpr int COST = M == 4 ? (T2 == 8 ? 20 : 16) : 30;
     __host__ __device__ static constexpr int dx(int lane) { return M == 4 ? (lane >> 2) & 3 : lane / 5; }
     __host__ __device__ static constexpr int dy(int lane) { return M == 4 ? lane & 3 : lane % 5; }
     __host__ __device__ static constexpr int half(int lane) { return M == 4 ? lane >> 4 : 0; }
@@ -2000,7 +2002,8 @@ __device__ __forceinline__ void fx_tile(const Record<float> *__restrict__ rec, c
         return w3 * fminf(static_cast<float>(M * M) * static_cast<float>(rowmax), static_cast<float>(n));
     };
     uint32_t reached = total;  // particles in cells of the reach
-    if (sshift > 0 && T2 + C::HL + C::HR < ng && min(M * M * s_rowmax, total) > 256u) {
+    constexpr bool RUNS = T2 >= 16;  // smaller tiles have one cell a key (plan_assign)
+    if (RUNS && sshift > 0 && T2 + C::HL + C::HR < ng && min(M * M * s_rowmax, total) > 256u) {
         // Keys of several cells: the ranges hold particles below and above the reach too. Up to
         // 256 the bound does not matter (tile_scales); above, the scale must be that of the
         // reach. It is where the runs inside the tile alone give the same power of two (and
@@ -2175,7 +2178,7 @@ __device__ __forceinline__ void fx_tile(const Record<float> *__restrict__ rec, c
                         const int b0 = first_node<M, C::HL, C::HR, T0>(u[k].x, packed & 1023, t0, ng);
                         const int b1 = first_node<M, C::HL, C::HR, T1>(u[k].y, (packed >> 10) & 1023, t1, ng);
                         const int b2 = first_node<M, C::HL, C::HR, T2>(u[k].z, (packed >> 20) & 1023, t2, ng);
-                        const bool reaches = (M % 2 == 0 && sshift == 0) || (b0 > -M && b0 < T0 && b1 > -M && b1 < T1 && b2 > -M && b2 < T2);
+                        const bool reaches = (M % 2 == 0 && (!RUNS || sshift == 0)) || (b0 > -M && b0 < T0 && b1 > -M && b1 < T1 && b2 > -M && b2 < T2);
                         const int g = (b0 * PX + b1 * RW + b2) & 31;
                         if (reaches) key[k] = g | static_cast<int>(atomicAdd(&s_bank[g], 1u) << 5);
                     }
